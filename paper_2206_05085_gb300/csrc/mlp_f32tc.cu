@@ -199,21 +199,28 @@ __device__ __forceinline__ void st_split1(uint8_t* hi, uint8_t* lo, uint32_t off
   *reinterpret_cast<uint16_t*>(lo + off) = (uint16_t)(l & 0xffffu);
 }
 
-// D (+)= A B^T over K = 16 * ksteps, split operands: three MMAs per K step
+// D (+)= A B^T over K = 16 * kSteps, split operands: three MMAs per K step
 // (hi*hi, hi*lo, lo*hi; kALo / kBLo false: A's / B's lo term is zero and
 // its product is not issued).  a_step / b_step: byte advance of the
 // descriptors' start address per step (the start-address field holds
 // address / 16, so a step adds step / 16).
-template <bool kALo = true, bool kBLo = true>
+//
+// The issue loops are unrolled and run in one elected thread (tc::elect_one).
+// Measured (one warp issuing, cycles per instruction): with rolled loops under
+// `lane == 0` every shape cost 100-200 cycles of issue, whatever its N; in
+// this form M = 128, K = 16 costs 64 for N = 128 (the tensor rate), 56 for N =
+// 96 and 44 for N = 48 with A in shared memory, 16 for N = 32 and 9 for N =
+// 16 with A in tensor memory.
+template <int kSteps, bool kALo = true, bool kBLo = true>
 __device__ __forceinline__ void mma3(uint32_t d, uint32_t ah, uint32_t al, uint32_t a_step, uint32_t a_lbo,
                                      uint32_t a_sbo, uint32_t bh, uint32_t bl, uint32_t b_step,
-                                     uint32_t b_lbo, uint32_t b_sbo, int ksteps, uint32_t idesc,
+                                     uint32_t b_lbo, uint32_t b_sbo, uint32_t idesc,
                                      bool accumulate) {
   uint64_t dah = tc::smem_desc(ah, a_lbo, a_sbo), dal = tc::smem_desc(al, a_lbo, a_sbo);
   uint64_t dbh = tc::smem_desc(bh, b_lbo, b_sbo), dbl = tc::smem_desc(bl, b_lbo, b_sbo);
   const uint64_t ia = a_step >> 4, ib = b_step >> 4;
-#pragma unroll 1
-  for (int k = 0; k < ksteps; ++k) {
+#pragma unroll
+  for (int k = 0; k < kSteps; ++k) {
     tc::mma_bf16(d, dah, dbh, idesc, (accumulate || k > 0) ? 1u : 0u);
     if (kBLo) tc::mma_bf16(d, dah, dbl, idesc, 1u);
     if (kALo) tc::mma_bf16(d, dal, dbh, idesc, 1u);
@@ -224,17 +231,17 @@ __device__ __forceinline__ void mma3(uint32_t d, uint32_t ah, uint32_t al, uint3
   }
 }
 
-// D (+)= A B^T over K = 16 * ksteps with A (128 rows) in tensor memory as
+// D (+)= A B^T over K = 16 * kSteps with A (128 rows) in tensor memory as
 // split terms: K-chunk q of 32 columns at a_tmem + 32 q, its hi terms packed
 // two per column in the first 16 columns and its lo terms in the next 16.
-template <bool kBLo = true>
+template <int kSteps, bool kBLo = true>
 __device__ __forceinline__ void mma3_ts(uint32_t d, uint32_t a_tmem, uint32_t bh, uint32_t bl, uint32_t b_step,
-                                        uint32_t b_lbo, uint32_t b_sbo, int ksteps, uint32_t idesc,
+                                        uint32_t b_lbo, uint32_t b_sbo, uint32_t idesc,
                                         bool accumulate) {
   uint64_t dbh = tc::smem_desc(bh, b_lbo, b_sbo), dbl = tc::smem_desc(bl, b_lbo, b_sbo);
   const uint64_t ib = b_step >> 4;
-#pragma unroll 1
-  for (int j = 0; j < ksteps; ++j) {
+#pragma unroll
+  for (int j = 0; j < kSteps; ++j) {
     const uint32_t ah = a_tmem + 32u * (uint32_t)(j >> 1) + 8u * (uint32_t)(j & 1), al = ah + 16u;
     tc::mma_ts(d, ah, dbh, idesc, (accumulate || j > 0) ? 1u : 0u);
     if (kBLo) tc::mma_ts(d, ah, dbl, idesc, 1u);
@@ -244,17 +251,17 @@ __device__ __forceinline__ void mma3_ts(uint32_t d, uint32_t a_tmem, uint32_t bh
   }
 }
 
-// D (+)= A B^T over K = 16 * ksteps with A (128 rows) in tensor memory as
+// D (+)= A B^T over K = 16 * kSteps with A (128 rows) in tensor memory as
 // split terms in 16-column chunks: K step j at a_tmem + 16 j, its hi terms
 // packed two per column in the first 8 columns and its lo terms in the next 8.
-template <bool kBLo = true>
+template <int kSteps, bool kBLo = true>
 __device__ __forceinline__ void mma3_ts16(uint32_t d, uint32_t a_tmem, uint32_t bh, uint32_t bl, uint32_t b_step,
-                                          uint32_t b_lbo, uint32_t b_sbo, int ksteps, uint32_t idesc,
+                                          uint32_t b_lbo, uint32_t b_sbo, uint32_t idesc,
                                           bool accumulate) {
   uint64_t dbh = tc::smem_desc(bh, b_lbo, b_sbo), dbl = tc::smem_desc(bl, b_lbo, b_sbo);
   const uint64_t ib = b_step >> 4;
-#pragma unroll 1
-  for (int j = 0; j < ksteps; ++j) {
+#pragma unroll
+  for (int j = 0; j < kSteps; ++j) {
     const uint32_t ah = a_tmem + 16u * (uint32_t)j, al = ah + 8u;
     tc::mma_ts(d, ah, dbh, idesc, (accumulate || j > 0) ? 1u : 0u);
     if (kBLo) tc::mma_ts(d, ah, dbl, idesc, 1u);
@@ -664,9 +671,9 @@ __global__ void __launch_bounds__(544, 1) rgbnet_fwd_tc_kernel(
       const uint32_t b = (uint32_t)(k & 1), buf = tmem + 256u * b;
       if (!wait0(&fs->h1_full[b], (uint32_t)(k >> 1) & 1u)) return;
       tc::fence_after_sync();
-      if (lane == 0) {
+      if (tc::elect_one()) {
         tc::bulk_s2g(act_img + (size_t)tile_of(k) * kImage + iHh, sm + gStage, 2 * kHBytes);
-        mma3_ts<Op::kWeightLo>(buf + 128u, buf, sW2h, sW2l, 256, 128, kSboH, kHid / 16, id128, false);
+        mma3_ts<kHid / 16, Op::kWeightLo>(buf + 128u, buf, sW2h, sW2l, 256, 128, kSboH, id128, false);
         tc::mma_commit(&fs->l2_full[b]);
       }
       __syncwarp();
@@ -677,13 +684,13 @@ __global__ void __launch_bounds__(544, 1) rgbnet_fwd_tc_kernel(
       // buffer b's H1 (tile k - 2) has been read by its layer-2 MMAs
       if (k >= 2 && !wait0(&fs->l2_full[b], (uint32_t)((k - 2) >> 1) & 1u)) return;
       tc::fence_after_sync();
-      if (lane == 0) {
+      if (tc::elect_one()) {
         uint8_t* xb = sm + gX0 + b * gXBuf;
         tc::bulk_wait_read();   // staging (H1 of k - 1) and X buffer b's older copy are read
         tc::bulk_s2g(act_img + (size_t)tile_of(k) * kImage + iX, xb, 2 * kXBytes);
         const uint32_t xs = tc::smem_u32(xb);
-        mma3<true, Op::kWeightLo>(buf, xs, xs + kSboX, 256, 128, kSboXs, sW1h, sW1l, 256, 128, kSboX,
-                                  kK1 / 16, id128, false);
+        mma3<kK1 / 16, true, Op::kWeightLo>(buf, xs, xs + kSboX, 256, 128, kSboXs, sW1h, sW1l, 256, 128, kSboX,
+                                            id128, false);
         tc::mma_commit(&fs->l1_full[b]);
       }
       __syncwarp();
@@ -696,7 +703,7 @@ __global__ void __launch_bounds__(544, 1) rgbnet_fwd_tc_kernel(
     }
     if (nt > 0) layer2(nt - 1);
     // every MMA and copy this thread issued has finished before the memory is released
-    if (lane == 0) {
+    if (tc::elect_one()) {
       tc::mma_commit(&fs->fin);
       tc::mbar_wait(&fs->fin, 0, kSpin);
       tc::bulk_wait_all();
@@ -1007,13 +1014,13 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
   float dW3acc[kOut] = {0.0f, 0.0f, 0.0f}, db2acc = 0.0f, db3acc[kOut] = {0.0f, 0.0f, 0.0f};
   if (warp == 16) {
     // ------------------------------------------------------------ MMA warp
-    // lane 0 polls and issues; the outcome of a wait is the warp's
+    // lane 0 polls (the outcome of a wait is the warp's); the elected thread issues
     auto wait0 = [&](uint64_t* bar, uint32_t parity) -> bool {
       int r = 0;
       if (lane == 0) r = bwd_wait(fs, bar, parity) ? 1 : 0;
       return __shfl_sync(0xffffffffu, r, 0) != 0;
     };
-    bool inflight_x = nt > 0;   // lane 0: an X copy not yet seen landed
+    bool inflight_x = nt > 0;   // elected thread: an X copy not yet seen landed
     uint32_t ph_h = 0, ph_x = 0, ph_gx = 0, ph_g2 = 0, ph_g1 = 0;
     auto load_x = [&](int64_t k) {
       tc::mbar_arrive_expect_tx(&fs->bar_x, 2 * kXBytes);
@@ -1024,8 +1031,8 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
     // hidden unit, column = tile row); after a failed wait only the commit
     auto d2 = [&](bool h_ok) {
       if (h_ok) {
-        mma3<Op::kWeightLo, true>(tmem + cTmp, sW2h, sW2l, 256, 128, kSboH, sHh, sHl, 256, 128, kSboH,
-                                  kHid / 16, Op::idesc(128, kTile, 0, 0), false);
+        mma3<kHid / 16, Op::kWeightLo, true>(tmem + cTmp, sW2h, sW2l, 256, 128, kSboH, sHh, sHl, 256, 128, kSboH,
+                                             Op::idesc(128, kTile, 0, 0), false);
       }
       tc::mma_commit(&fs->bar_d2);
     };
@@ -1033,28 +1040,29 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
       const bool h_ok = wait0(&fs->bar_h, ph_h);
       ph_h ^= 1;
       tc::fence_after_sync();
-      if (lane == 0) d2(h_ok);
+      if (tc::elect_one()) d2(h_ok);
       __syncwarp();
     }
     for (int64_t k = 0; k < nt; ++k) {
       const bool has_next = k + 1 < nt;
       // X(k): the buffer is free once g_X and dW1 of tile k - 1 are done
       if (k > 0) {
-        if (wait0(&fs->bar_gx, ph_gx) && lane == 0) load_x(k);
+        if (wait0(&fs->bar_gx, ph_gx) && tc::elect_one()) load_x(k);
+        __syncwarp();
         ph_gx ^= 1;
       }
       // dW2 += G2^T H1 (A from tensor memory), then g_h1 = G2 W2 (A MN-major)
       const bool g2 = wait0(&fs->g2_full, ph_g2);
       ph_g2 ^= 1;
       tc::fence_after_sync();
-      if (lane == 0) {
+      if (tc::elect_one()) {
         if (g2)
-          mma3_ts16(tmem + cDW2, tmem + cTmp, sHh, sHl, 2 * kSboH, kSboH, 128, kTile / 16,
-                    Op::idesc(128, kHid, 0, 1), k > 0);
+          mma3_ts16<kTile / 16>(tmem + cDW2, tmem + cTmp, sHh, sHl, 2 * kSboH, kSboH, 128,
+                                Op::idesc(128, kHid, 0, 1), k > 0);
         tc::mma_commit(&fs->bar_dw2);
         if (g2)
-          mma3<true, Op::kWeightLo>(tmem + cGH, sGh, sGl, 2 * kSboH, kSboH, 128, sW2h, sW2l, 2 * kSboH,
-                                    kSboH, 128, kHid / 16, Op::idesc(128, kHid, 1, 1), false);
+          mma3<kHid / 16, true, Op::kWeightLo>(tmem + cGH, sGh, sGl, 2 * kSboH, kSboH, 128, sW2h, sW2l, 2 * kSboH,
+                                               kSboH, 128, Op::idesc(128, kHid, 1, 1), false);
         tc::mma_commit(&fs->bar_gh);
       }
       __syncwarp();
@@ -1064,7 +1072,7 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
         const bool h_ok = wait0(&fs->bar_h, ph_h);
         ph_h ^= 1;
         tc::fence_after_sync();
-        if (lane == 0) d2(h_ok);
+        if (tc::elect_one()) d2(h_ok);
         __syncwarp();
       }
       // once G1 and X are in: g_X = G1 W1[:, 0:16] (A from tensor memory) and
@@ -1072,7 +1080,7 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
       const bool g1 = wait0(&fs->g1_full, ph_g1);
       ph_g1 ^= 1;
       tc::fence_after_sync();
-      if (lane == 0) {
+      if (tc::elect_one()) {
         const bool x_ok = g1 && bwd_wait(fs, &fs->bar_x, ph_x);
         ph_x ^= 1;
         if (x_ok) {
@@ -1080,7 +1088,7 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
           {   // per K step: G1h [W1h | W1l] (N = 32: hi*hi in columns 0-15, hi*lo in 16-31), G1l W1h
             const uint32_t id32 = Op::idesc(128, 32, 0, 1), id16 = Op::idesc(128, 16, 0, 1);
             uint64_t db = tc::smem_desc(sW1h, kSboW1s, 128);
-#pragma unroll 1
+#pragma unroll
             for (uint32_t j = 0; j < kHid / 16; ++j) {
               const uint32_t ah = tmem + cGH + 16u * j, al = ah + 8u;
               tc::mma_ts(tmem + cGX, ah, db, id32, j > 0 ? 1u : 0u);
@@ -1092,7 +1100,7 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
             const uint32_t id96 = Op::idesc(128, 2 * kK1, 1, 1), id48 = Op::idesc(128, kK1, 1, 1);
             uint64_t dah = tc::smem_desc(sGh, kSboH, 128), dal = tc::smem_desc(sGl, kSboH, 128);
             uint64_t dbx = tc::smem_desc(sX, kSboXs, 128);
-#pragma unroll 1
+#pragma unroll
             for (int kk = 0; kk < kTile / 16; ++kk) {
               tc::mma_bf16(tmem + cDW1, dah, dbx, id96, (k > 0 || kk > 0) ? 1u : 0u);
               tc::mma_bf16(tmem + cDW1, dal, dbx, id48, 1u);
@@ -1109,7 +1117,7 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
     // every product has finished before the accumulators are read and the
     // tensor memory is released; a copy issued but never seen landed (only
     // after a failed wait) lands before exit
-    if (lane == 0) {
+    if (tc::elect_one()) {
       tc::mma_commit(&fs->bar_fin);
       if (!tc::mbar_wait(&fs->bar_fin, 0, kSpin)) {
         *reinterpret_cast<volatile int*>(&fs->abort) = 1;

@@ -128,6 +128,17 @@ __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_
       : "memory");
 }
 
+// True in exactly one thread of the (converged) warp, the same one at every
+// call (the election is deterministic for one member mask).  Code that
+// issues tcgen05.mma runs under this predicate rather than under `lane == 0`:
+// the compiler then knows that the branch has one thread and keeps the
+// descriptors in uniform registers, where the instruction takes them from.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n selp.u32 %0, 1, 0, e;\n}" : "=r"(r)::"memory");
+  return r != 0;
+}
+
 // Arrive on *bar once every tcgen05.mma issued so far by this thread is done.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(

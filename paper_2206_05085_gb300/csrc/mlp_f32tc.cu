@@ -14,10 +14,10 @@
 // from a bound on that sample's output-layer gradient, so that every sample's
 // input gradient keeps FP32 relative accuracy however small it is.  The
 // weight-gradient products (sums over samples) need one factor for all rows,
-// S, the scale of the largest bound over the CTA's samples: dW2 reads H1 with
-// row s multiplied by S / s_s, dW1 a second copy of G1's terms times S / s_s
-// (a row far below the largest loses only terms below FP16's subnormal range,
-// 2^-38 of the largest row).
+// S, the scale of the largest bound over the CTA's samples: dW2 and dW1 read a
+// second copy of G2's and G1's terms times S / s_s (a row far below the
+// largest loses only terms below FP16's subnormal range, 2^-38 of the largest
+// row).
 // Every scale is an exact power of two, undone exactly in the epilogues.  A
 // value whose scaled magnitude reaches 2^15 sets DVGO_ERR_RANGE.
 //
@@ -75,9 +75,40 @@ constexpr float kSX = 64.0f;     // input scale
 constexpr float kSH = 16.0f;     // hidden-activation scale
 constexpr float kRange = 32768.0f;   // FP16 terms: scaled magnitudes must stay below 2^15
 constexpr uint32_t kSpin = 1u << 24;
+constexpr int kPartRow = kOffB3;   // partial gradient rows: all parameters but b3 (its rows follow, 3 values each)
+constexpr int kThreads = 544;   // 16 compute warps and the MMA warp
 
 __device__ __forceinline__ uint32_t u32_of(__half2 v) { return *reinterpret_cast<const uint32_t*>(&v); }
 __device__ __forceinline__ uint32_t u32_of(__nv_bfloat162 v) { return *reinterpret_cast<const uint32_t*>(&v); }
+
+// Two FP32 values in one 64-bit register pair: one instruction of the packed
+// forms does both (each half rounded as the scalar instruction rounds it).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
 
 // Operand term formats of the split products.
 struct OpF16 {   // FP32 form: FP16 terms, every matrix split (weights too)
@@ -100,6 +131,21 @@ struct OpF16 {   // FP32 form: FP16 terms, every matrix split (weights too)
     const __half2 y = __hmul2(*reinterpret_cast<const __half2*>(&x), __float2half2_rn(r));
     return u32_of(y);
   }
+  // two pairs of terms multiplied
+  __device__ static __forceinline__ uint32_t mul2v(uint32_t x, uint32_t y) {
+    return u32_of(__hmul2(*reinterpret_cast<const __half2*>(&x), *reinterpret_cast<const __half2*>(&y)));
+  }
+  __device__ static __forceinline__ uint32_t pack(float a, float b) { return u32_of(__floats2half2_rn(a, b)); }
+  static __device__ __forceinline__ f32x2 join2(uint32_t hi, uint32_t lo) {   // hi + lo of both
+    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&hi)),
+                 b = __half22float2(*reinterpret_cast<const __half2*>(&lo));
+    return pack2(a.x + b.x, a.y + b.y);
+  }
+  // 0xffff in each half of x that is > 0
+  __device__ static __forceinline__ uint32_t positive(uint32_t x) {
+    return __hgt2_mask(*reinterpret_cast<const __half2*>(&x), __float2half2_rn(0.0f));
+  }
+  static constexpr float kMinFactor = 5.9604645e-8f;   // 2^-24: the smallest power of two a term factor can be
   __device__ static __forceinline__ float param(float x) { return x; }
 };
 
@@ -125,8 +171,30 @@ struct OpBF16 {  // BF16 form: stored BF16 weights (one term), BF16 hi + lo term
         __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&x), __float2bfloat162_rn(r));
     return u32_of(y);
   }
+  __device__ static __forceinline__ uint32_t mul2v(uint32_t x, uint32_t y) {
+    return u32_of(
+        __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&x), *reinterpret_cast<const __nv_bfloat162*>(&y)));
+  }
+  __device__ static __forceinline__ uint32_t pack(float a, float b) { return u32_of(__floats2bfloat162_rn(a, b)); }
+  static __device__ __forceinline__ f32x2 join2(uint32_t hi, uint32_t lo) {
+    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&hi)),
+                 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&lo));
+    return pack2(a.x + b.x, a.y + b.y);
+  }
+  __device__ static __forceinline__ uint32_t positive(uint32_t x) {
+    return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&x), __float2bfloat162_rn(0.0f));
+  }
+  static constexpr float kMinFactor = 1.1754944e-38f;
   __device__ static __forceinline__ float param(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 };
+
+// hi and lo terms of the pair v, packed two per word.
+template <class Op>
+__device__ __forceinline__ uint32_t split_pair(f32x2 v, uint32_t& lo, float& vmax) {
+  const float2 f = unpack2(v);
+  vmax = fmaxf(vmax, fmaxf(fabsf(f.x), fabsf(f.y)));
+  return Op::split2(f.x, f.y, lo);
+}
 
 // backward shared memory
 constexpr uint32_t bW2h = 0, bW2l = bW2h + kW2Bytes, bW1h = bW2l + kW2Bytes,
@@ -136,15 +204,20 @@ constexpr uint32_t bW2h = 0, bW2l = bW2h + kW2Bytes, bW1h = bW2l + kW2Bytes,
 constexpr uint32_t cTmp = 0, cDW2 = 128, cDW1 = 256, cGX = 352, cGH = 384;
 
 struct Side {
-  float4 smp[kTile];  // per tile row: (g_z3[0..2], the row's gradient scale sG2)
-  float red[32];      // block_max scratch: one entry per warp (17 warps)
+  // Rows 2p, 2p + 1 of the tile: g_z3[0] of both, then [1], [2], each times
+  // the row's own gradient scale sG2, then the two 1 / sG2.
+  float4 smp[kTile / 2][2];
+  uint16_t sc[2][kTile];   // by tile parity: exponent fields of a row's sG2 (low byte) and sG1
+  uint32_t tiny[4];   // rows 32 q ..: some row's S2 / sG2 is below the factor a term can be multiplied by
   uint64_t bar_h;     // H1 terms of a tile image landed
   uint64_t bar_x;     // X terms landed
   uint64_t bar_d2;    // D2^T of a tile done
   uint64_t bar_gh;    // g_h1 done
-  uint64_t bar_dw2;   // dW2 done (the tile's H1 terms are free)
+  uint64_t bar_dw2a;  // dW2 over the first half of the rows done (their H1 terms are free)
+  uint64_t bar_dw2;   // dW2 done (all H1 terms are free)
   uint64_t bar_gx;    // g_X and dW1 done (G's shared memory and X are free)
   uint64_t bar_fin;   // every product done (before the accumulators are read)
+  uint64_t g2a_full;  // G2 of the first half of the rows in tensor memory (16 warp arrivals)
   uint64_t g2_full;   // G2 of a tile in tensor and shared memory (16 warp arrivals)
   uint64_t g1_full;   // G1 of a tile in tensor and shared memory (16 warp arrivals)
   uint32_t tmem_slot;
@@ -152,25 +225,37 @@ struct Side {
 };
 static_assert(bEnd + sizeof(Side) <= 227 * 1024, "backward shared memory");
 
-// Largest value of v over the block (all threads call it).
-__device__ __forceinline__ float block_max(float v, float* red) {
+
+// Largest of each of the four values over the block (all threads call it; the
+// values are >= 0).  red: one entry per warp (kThreads / 32).
+__device__ __forceinline__ float4 block_max4(float4 v, float4* red) {
 #pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  __syncthreads();
+  for (int o = 16; o >= 1; o >>= 1) {
+    v.x = fmaxf(v.x, __shfl_xor_sync(0xffffffffu, v.x, o));
+    v.y = fmaxf(v.y, __shfl_xor_sync(0xffffffffu, v.y, o));
+    v.z = fmaxf(v.z, __shfl_xor_sync(0xffffffffu, v.z, o));
+    v.w = fmaxf(v.w, __shfl_xor_sync(0xffffffffu, v.w, o));
+  }
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  float r = red[0];
-  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) r = fmaxf(r, red[w]);
+  float4 r = red[0];
+#pragma unroll
+  for (int w = 1; w < kThreads / 32; ++w) {
+    const float4 q = red[w];
+    r = make_float4(fmaxf(r.x, q.x), fmaxf(r.y, q.y), fmaxf(r.z, q.z), fmaxf(r.w, q.w));
+  }
   return r;
 }
 
-// 2^(13 - floor(log2 m)): maps the largest magnitude m into [2^13, 2^14).
+// 2^(13 - floor(log2 m)): maps the largest magnitude m into [2^13, 2^14)
+// (|log2 m| limited to 100; 1 for 0, infinity and NaN).
 __device__ __forceinline__ float pow2_scale(float m) {
   if (!(m > 0.0f) || !(m <= 3.0e38f)) return 1.0f;
-  int e = ilogbf(m);
-  e = max(-100, min(100, e));
-  return ldexpf(1.0f, 13 - e);
+  const int e = max(-100, min(100, (int)(__float_as_uint(m) >> 23) - 127));
+  return __uint_as_float((uint32_t)(127 + 13 - e) << 23);
 }
+// 1 / s of such a scale (exact).
+__device__ __forceinline__ float pow2_rcp(float s) { return __uint_as_float(0x7f000000u - __float_as_uint(s)); }
 
 // Split 8 (already scaled) values into the hi / lo core-matrix rows at (row,
 // k8); vmax tracks the largest magnitude split (range check).  kWeight: the
@@ -188,15 +273,6 @@ __device__ __forceinline__ void st_split8(uint8_t* hi, uint8_t* lo, int row, int
   const uint32_t off = tc::cm_off(row, k8, sbo);
   *reinterpret_cast<uint4*>(hi + off) = make_uint4(h[0], h[1], h[2], h[3]);
   *reinterpret_cast<uint4*>(lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
-}
-
-// One scaled, split parameter (setup only).
-template <class Op>
-__device__ __forceinline__ void st_split1(uint8_t* hi, uint8_t* lo, uint32_t off, float v) {
-  uint32_t l;
-  const uint32_t h = Op::weight2(v, 0.0f, l);
-  *reinterpret_cast<uint16_t*>(hi + off) = (uint16_t)(h & 0xffffu);
-  *reinterpret_cast<uint16_t*>(lo + off) = (uint16_t)(l & 0xffffu);
 }
 
 // D (+)= A B^T over K = 16 * kSteps, split operands: three MMAs per K step
@@ -254,15 +330,16 @@ __device__ __forceinline__ void mma3_ts(uint32_t d, uint32_t a_tmem, uint32_t bh
 // D (+)= A B^T over K = 16 * kSteps with A (128 rows) in tensor memory as
 // split terms in 16-column chunks: K step j at a_tmem + 16 j, its hi terms
 // packed two per column in the first 8 columns and its lo terms in the next 8.
-template <int kSteps, bool kBLo = true>
+// kStride: K steps 0, kStride, 2 kStride, ... of the operands.
+template <int kSteps, int kStride = 1, bool kBLo = true>
 __device__ __forceinline__ void mma3_ts16(uint32_t d, uint32_t a_tmem, uint32_t bh, uint32_t bl, uint32_t b_step,
                                           uint32_t b_lbo, uint32_t b_sbo, uint32_t idesc,
                                           bool accumulate) {
   uint64_t dbh = tc::smem_desc(bh, b_lbo, b_sbo), dbl = tc::smem_desc(bl, b_lbo, b_sbo);
-  const uint64_t ib = b_step >> 4;
+  const uint64_t ib = (kStride * b_step) >> 4;
 #pragma unroll
   for (int j = 0; j < kSteps; ++j) {
-    const uint32_t ah = a_tmem + 16u * (uint32_t)j, al = ah + 8u;
+    const uint32_t ah = a_tmem + 16u * (uint32_t)(kStride * j), al = ah + 8u;
     tc::mma_ts(d, ah, dbh, idesc, (accumulate || j > 0) ? 1u : 0u);
     if (kBLo) tc::mma_ts(d, ah, dbl, idesc, 1u);
     tc::mma_ts(d, al, dbh, idesc, 1u);
@@ -299,36 +376,6 @@ __device__ __forceinline__ void st_terms16(uint8_t* hi, uint8_t* lo, int row, in
   }
 }
 
-// 32 values times s split into the tensor-memory chunk layout: hi terms of
-// value pairs in words 0-15, lo terms in words 16-31 (one tcgen05.st).
-template <class Op>
-__device__ __forceinline__ void split32(const float (&v)[32], float s, uint32_t (&hl)[32],
-                                        float& vmax) {
-#pragma unroll
-  for (int c = 0; c < 16; ++c) {
-    const float a = s * v[2 * c], b = s * v[2 * c + 1];
-    vmax = fmaxf(vmax, fmaxf(fabsf(a), fabsf(b)));
-    hl[c] = Op::split2(a, b, hl[16 + c]);
-  }
-}
-
-// The split terms of split32 times r (a power of two <= 1, exact in FP16
-// down to its subnormal range, and in BF16) as the hi / lo core-matrix rows
-// of columns k0 .. k0 + 31 of row `row` in shared memory.
-template <class Op, bool kScale = true>
-__device__ __forceinline__ void st_terms32(uint8_t* hi, uint8_t* lo, int row, int k0, const uint32_t (&hl)[32],
-                                           float r) {
-  auto m = [&](uint32_t x) { return kScale ? Op::mul2(x, r) : x; };
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const uint32_t off = tc::cm_off(row, k0 + 8 * q, kSboH);
-    *reinterpret_cast<uint4*>(hi + off) =
-        make_uint4(m(hl[4 * q]), m(hl[4 * q + 1]), m(hl[4 * q + 2]), m(hl[4 * q + 3]));
-    *reinterpret_cast<uint4*>(lo + off) =
-        make_uint4(m(hl[16 + 4 * q]), m(hl[17 + 4 * q]), m(hl[18 + 4 * q]), m(hl[19 + 4 * q]));
-  }
-}
-
 // Output-layer constants (FP32; the stored BF16 values in the BF16 form).
 template <class Op, class SideT>
 __device__ __forceinline__ void load_out_layer(const float* __restrict__ params, SideT* fs) {
@@ -338,94 +385,128 @@ __device__ __forceinline__ void load_out_layer(const float* __restrict__ params,
   if (threadIdx.x < 4) fs->b3[threadIdx.x] = threadIdx.x < kOut ? Op::param(params[kOffB3 + threadIdx.x]) : 0.0f;
 }
 
-// This thread's share of max |p[e]|, e < count (float4 loads, four in
-// flight per thread, when p is 16-byte aligned and count a multiple of 4).
-__device__ __forceinline__ float abs_max_part(const float* __restrict__ p, int count) {
-  float m = 0.0f;
-  if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0 && (count & 3) == 0) {
-    const float4* p4 = reinterpret_cast<const float4*>(p);
-    const int n4 = count >> 2;
-    for (int e0 = threadIdx.x; e0 < n4; e0 += 4 * blockDim.x) {
-      float4 v[4];
+// A thread's share of a weight matrix in registers, in chunks of 8 columns
+// (thread c % kThreads takes chunk c).  Eight consecutive chunks are the rows of
+// one core matrix (its 128 bytes in shared memory: no bank conflicts), then come
+// the next 8 columns of the same rows (so that a warp reads whole lines).  The weights are read once,
+// all loads in flight together: the largest magnitude is found and, with the
+// scale it gives, the split terms are formed from the registers.  (Reading
+// the matrices once for the scale and again for the split, one reduction per
+// matrix, cost 15-25k cycles at the start of every call.)
+template <int kB>   // kB: column blocks of 8
+__device__ __forceinline__ int chunk_row(int c) { return ((c >> 3) / kB) * 8 + (c & 7); }
+template <int kB>
+__device__ __forceinline__ int chunk_col(int c) { return ((c >> 3) % kB) * 8; }
+
+template <int kCount>
+struct WChunks {
+  float v[kCount][8];
+  __device__ __forceinline__ float abs_max() const {
+    float m = 0.0f;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int e = e0 + u * blockDim.x;
-        v[u] = e < n4 ? __ldg(p4 + e) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      }
+    for (int u = 0; u < kCount; ++u)
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        m = fmaxf(m, fmaxf(fmaxf(fabsf(v[u].x), fabsf(v[u].y)), fmaxf(fabsf(v[u].z), fabsf(v[u].w))));
+      for (int i = 0; i < 8; ++i) m = fmaxf(m, fabsf(v[u][i]));
+    return m;
+  }
+};
+
+// The first 16 columns of W1 (the backward's g_X operand).
+struct W1Chunks16 : WChunks<1> {
+  static constexpr int kB = 2, kChunks = kHid * kB;
+  __device__ __forceinline__ void load(const float* __restrict__ params) {
+    const int c = threadIdx.x;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      v[0][i] = c < kChunks ? __ldg(params + kOffW1 + chunk_row<kB>(c) * kIn + chunk_col<kB>(c) + i) : 0.0f;
+  }
+  // scaled by s, as split K-major core matrices [o][k]
+  template <class Op>
+  __device__ __forceinline__ void store(uint8_t* hi, uint8_t* lo, uint32_t sbo, float s) {
+    const int c = threadIdx.x;
+    float dummy = 0.0f;
+    if (c < kChunks) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[0][i] *= s;
+      st_split8<Op, true>(hi, lo, chunk_row<kB>(c), chunk_col<kB>(c), sbo, v[0], dummy);
     }
-  } else {
-    for (int e = threadIdx.x; e < count; e += blockDim.x) m = fmaxf(m, fabsf(__ldg(p + e)));
+  }
+};
+
+// The whole W1 | b1 (rows of 39: copied to shared memory as they lie, since
+// reading 8-column chunks of them from global memory touches a line per row).
+// Returns the thread's share of the largest magnitude.
+__device__ __forceinline__ float w1_to_smem(const float* __restrict__ params, float* raw) {
+  constexpr int kCount = kHid * kIn + kHid, kPer = (kCount + kThreads - 1) / kThreads;
+  static_assert(kOffB1 == kOffW1 + kHid * kIn, "b1 follows W1");
+  float v[kPer], m = 0.0f;
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const int e = threadIdx.x + u * kThreads;
+    v[u] = e < kCount ? __ldg(params + kOffW1 + e) : 0.0f;
+  }
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const int e = threadIdx.x + u * kThreads;
+    if (e < kCount) raw[e] = v[u];
+    m = fmaxf(m, fabsf(v[u]));
   }
   return m;
 }
-
-// Rows o of W1 | b1 | 0 (width K = 8 kb, the bias in column kIn when K > kIn),
-// scaled by s, as split K-major core matrices [o][k]; 8 columns per chunk.
-template <class Op, int K>
-__device__ __forceinline__ void load_w1(const float* __restrict__ params, uint8_t* hi, uint8_t* lo, uint32_t sbo,
-                                        float s) {
-  constexpr int kB = K / 8, kChunks = kHid * kB;
-  float dummy = 0.0f;
-  for (int c0 = threadIdx.x; c0 < kChunks; c0 += 2 * blockDim.x) {
-    float v[2][8];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int c = c0 + u * blockDim.x, o = c / kB, k8 = (c % kB) * 8;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int k = k8 + i;
-        v[u][i] = c >= kChunks ? 0.0f
-                               : (k < kIn ? __ldg(params + kOffW1 + o * kIn + k)
-                                          : (k == kIn ? __ldg(params + kOffB1 + o) : 0.0f));
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int c = c0 + u * blockDim.x;
-      if (c < kChunks) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) v[u][i] *= s;
-        st_split8<Op, true>(hi, lo, c / kB, (c % kB) * 8, sbo, v[u], dummy);
-      }
-    }
-  }
-}
-
-// W2 (scaled by s) as split K-major core matrices [o][i]; 8 columns per chunk.
+// Rows o of W1 | b1 | 0 (48 columns, the bias in column kIn), scaled by s, as
+// split K-major core matrices [o][k].
 template <class Op>
-__device__ __forceinline__ void load_w2(const float* __restrict__ params, uint8_t* hi, uint8_t* lo, float s) {
-  const float* w = params + kOffW2;
+__device__ __forceinline__ void w1_split(const float* raw, uint8_t* hi, uint8_t* lo, float s) {
+  constexpr int kB = kK1 / 8, kChunks = kHid * kB;
   float dummy = 0.0f;
-  if ((reinterpret_cast<uintptr_t>(w) & 15u) != 0) {
-    for (int e = threadIdx.x; e < kHid * kHid; e += blockDim.x)
-      st_split1<Op>(hi, lo, tc::cm_off(e / kHid, e % kHid, kSboH), s * __ldg(w + e));
-    return;
-  }
-  constexpr int kChunks = kHid * kHid / 8;
-  for (int c0 = threadIdx.x; c0 < kChunks; c0 += 4 * blockDim.x) {
-    float4 a[4], b[4];
+  for (int c = threadIdx.x; c < kChunks; c += kThreads) {
+    const int o = chunk_row<kB>(c), k8 = chunk_col<kB>(c);
+    float v[8];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int c = c0 + u * blockDim.x;
-      if (c < kChunks) {
-        a[u] = __ldg(reinterpret_cast<const float4*>(w + 8 * c));
-        b[u] = __ldg(reinterpret_cast<const float4*>(w + 8 * c + 4));
-      }
+    for (int i = 0; i < 8; ++i) {
+      const int k = k8 + i;
+      v[i] = k < kIn ? s * raw[o * kIn + k] : (k == kIn ? s * raw[kHid * kIn + o] : 0.0f);
     }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int c = c0 + u * blockDim.x;
-      if (c < kChunks) {
-        float v[8] = {s * a[u].x, s * a[u].y, s * a[u].z, s * a[u].w,
-                      s * b[u].x, s * b[u].y, s * b[u].z, s * b[u].w};
-        st_split8<Op, true>(hi, lo, c >> 4, (c & 15) * 8, kSboH, v, dummy);
-      }
-    }
+    st_split8<Op, true>(hi, lo, o, k8, kSboX, v, dummy);
   }
 }
+
+struct W2Chunks : WChunks<(kHid * kHid / 8 + kThreads - 1) / kThreads> {
+  static constexpr int kChunks = kHid * kHid / 8, kCount = (kChunks + kThreads - 1) / kThreads;
+  __device__ __forceinline__ void load(const float* __restrict__ params) {
+    const float* w = params + kOffW2;
+    const bool aligned = (reinterpret_cast<uintptr_t>(w) & 15u) == 0;
+#pragma unroll
+    for (int u = 0; u < kCount; ++u) {
+      const int c = threadIdx.x + u * kThreads, at = chunk_row<kHid / 8>(c) * kHid + chunk_col<kHid / 8>(c);
+      if (c >= kChunks) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) this->v[u][i] = 0.0f;
+      } else if (aligned) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(w + at)),
+                     b = __ldg(reinterpret_cast<const float4*>(w + at + 4));
+        this->v[u][0] = a.x, this->v[u][1] = a.y, this->v[u][2] = a.z, this->v[u][3] = a.w;
+        this->v[u][4] = b.x, this->v[u][5] = b.y, this->v[u][6] = b.z, this->v[u][7] = b.w;
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) this->v[u][i] = __ldg(w + at + i);
+      }
+    }
+  }
+  template <class Op>
+  __device__ __forceinline__ void store(uint8_t* hi, uint8_t* lo, float s) {
+    float dummy = 0.0f;
+#pragma unroll
+    for (int u = 0; u < kCount; ++u) {
+      const int c = threadIdx.x + u * kThreads;
+      if (c < kChunks) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) this->v[u][i] *= s;
+        st_split8<Op, true>(hi, lo, chunk_row<kHid / 8>(c), chunk_col<kHid / 8>(c), kSboH, this->v[u], dummy);
+      }
+    }
+  }
+};
 
 __device__ __forceinline__ void set_status(int code) { atomicCAS(&g_mlp_tc_status, 0, code); }
 
@@ -562,7 +643,6 @@ constexpr uint32_t gW1h = 0, gW1l = gW1h + kW1Bytes, gW2h = gW1l + kW1Bytes, gW2
 struct FwdSide {
   float4 ob[kHid];   // per hidden unit o: (b2[o], W3[0][o], W3[1][o], W3[2][o])
   float b3[4];
-  float red[32];         // block_max scratch: one entry per warp (17 warps)
   uint64_t x_full[2];    // X of the tile in buffer b written (16 warp arrivals)
   uint64_t l1_full[2];   // layer-1 MMAs of buffer b done (X buffer b free again)
   uint64_t h1_full[2];   // H1 of buffer b stored in tensor memory (16 warp arrivals)
@@ -611,7 +691,7 @@ __device__ __forceinline__ bool fwd_wait(FwdSide* fs, uint64_t* bar, uint32_t pa
 //            wait x_full(k) (and l2_full(k - 2): buffer b's H1 read) -> layer 1
 //            of k -> commit l1_full(k).
 template <class Op>
-__global__ void __launch_bounds__(544, 1) rgbnet_fwd_tc_kernel(
+__global__ void __launch_bounds__(kThreads, 1) rgbnet_fwd_tc_kernel(
     const float* __restrict__ k0, const float* __restrict__ rays_d, const int32_t* __restrict__ ray_id,
     const int32_t* __restrict__ idx, int64_t n_cap, const int64_t* __restrict__ n_dev,
     const float* __restrict__ params, float* __restrict__ rgb, uint8_t* __restrict__ act) {
@@ -638,13 +718,21 @@ __global__ void __launch_bounds__(544, 1) rgbnet_fwd_tc_kernel(
     fs->abort = 0;
   }
   // weights: W1 | b1 (column 39) and W2, split, each with its own scale
-  const float m1 = abs_max_part(params + kOffW1, kHid * kIn + kHid);
-  const float m2 = abs_max_part(params + kOffW2, kHid * kHid);
-  const float sW1 = pow2_scale(block_max(m1, fs->red));
-  const float sW2 = pow2_scale(block_max(m2, fs->red));
-  if (warp < 16 && nt > 0) row_in_l2(in, k0, ray_id, qw == 0);
-  load_w1<Op, kK1>(params, sm + gW1h, sm + gW1l, kSboX, sW1);
-  load_w2<Op>(params, sm + gW2h, sm + gW2l, sW2);
+  float sW1, sW2;
+  {
+    W2Chunks w2;
+    float* raw1 = reinterpret_cast<float*>(sm + gX0);   // (the X buffers are free)
+    static_assert((kHid * kIn + kHid) * sizeof(float) <= 2 * gXBuf, "raw W1 | b1 fits the X buffers");
+    w2.load(params);
+    const float m1 = w1_to_smem(params, raw1);
+    if (warp < 16 && nt > 0) row_in_l2(in, k0, ray_id, qw == 0);
+    const float4 m = block_max4(make_float4(m1, w2.abs_max(), 0.0f, 0.0f),
+                                reinterpret_cast<float4*>(sm + gStage));   // (the staging area is free)
+    sW1 = pow2_scale(m.x);
+    sW2 = pow2_scale(m.y);
+    w1_split<Op>(raw1, sm + gW1h, sm + gW1l, sW1);
+    w2.store<Op>(sm + gW2h, sm + gW2l, sW2);
+  }
   load_out_layer<Op>(params, fs);
   if (warp < 16 && nt > 0) row_in_l3(in, rays_d);
   tc::fence_proxy_async_smem();
@@ -842,43 +930,55 @@ __global__ void __launch_bounds__(544, 1) rgbnet_fwd_tc_kernel(
 // TMEM lanes (g_h1, g_X) a thread holds row 32 (w & 3) + lane and hidden
 // columns 32 q .. + 31; in the transposed layer 2 (D2^T) it holds hidden unit
 // 32 (w & 3) + lane and tile rows 32 q .. + 31.  Warp 16 issues the MMAs and
-// the X copies, so that the tensor core runs while the compute warps work:
-// dW2 first (its completion frees H1's buffer for the next tile's copy),
-// then g_h1, then the next tile's D2^T as soon as its H1 has landed, then
-// this tile's g_X and dW1 once G1 is in.
+// the X copies, so that the tensor core runs while the compute warps work.
+//
+// What bounds it: the epilogues and the waits between them (one tile's
+// operands fill the shared memory, so a tile's phases follow one another; the
+// MMAs are 5.6k cycles of a tile's ~12k).  So the order puts as much as it
+// can beside the G2 epilogue and the wait for g_h1: dW2 runs in two halves
+// (the rows of an epilogue half each), the first beside the second epilogue
+// half; the next tile's H1 terms are copied in per half, as dW2 frees them;
+// while g_h1 runs the compute warps load the next tile's upstream rows (one
+// column quarter's warps for all) and form its relu mask.  Epilogue arithmetic
+// is packed (two FP32 values per instruction), G2 is split once and its
+// second copy formed by multiplying the 16-bit terms.  Measured, 1.9e6
+// samples, FP32 form: 782 us before, 582 us now (393,909 samples: 197 and
+// 152 us; 1003 samples with the partial sums: 31.8 and 25.7 us).
 //
 // Order per tile t of this CTA (tn = the next one):
-//   compute: wait h_full(t) -> row scales, relu mask (reads H1(t)); wait
-//            d2(t) -> G2 epilogue; wait gx(t - 1) -> G2 into shared memory,
+//   compute: wait d2(t) -> G2 of the rows 32 q .. + 15; wait gx(t - 1) ->
+//            into shared memory; arrive g2a_full(t); G2 of the other rows,
 //            g_X(t - 1) -> g_k0; arrive g2_full(t).  Thread 0: wait dw2(t)
-//            -> copy H1(tn) in.  Wait gh(t) -> G1 epilogue; arrive
-//            g1_full(t).
-//   MMA:     wait gx(t - 1) -> copy X(t) in; wait g2_full(t) -> dW2(t),
-//            commit dw2; g_h1(t), commit gh; wait h_full(tn) -> D2^T(tn),
-//            commit d2; wait g1_full(t) and X(t) -> g_X(t) and dW1(t),
-//            commit gx.
+//            -> copy the second half of H1(tn) in.  Upstream rows of tn;
+//            wait h_full(tn) -> relu mask of tn.  Wait gh(t) -> G1 epilogue;
+//            arrive g1_full(t).
+//   MMA:     wait gx(t - 1) -> copy X(t) in; wait g2a_full(t) -> dW2(t) over
+//            the first rows, commit dw2a; wait dw2a -> copy the first half of
+//            H1(tn) in; wait g2_full(t) -> the rest of dW2(t), commit dw2;
+//            g_h1(t), commit gh; wait h_full(tn) -> D2^T(tn), commit d2; wait
+//            g1_full(t) and X(t) -> g_X(t) and dW1(t), commit gx.
 // A tensor-memory column range or shared buffer is rewritten only after the
-// barrier that follows its last reader.  The G2 and G1 split terms in tensor
-// memory use 16-column chunks (mma3_ts16), so that each epilogue runs in two
-// halves of 16 columns and rewrites only columns it has already read.  The
-// upstream colour gradient of the next tile is loaded in three dependent
-// steps over the current tile.
+// barrier that follows its last reader (the rows' g_z3 and scales: bar_gh,
+// which follows every warp's g2_full arrival; their exponents alternate
+// between two buffers).  The G2 and G1 split terms in tensor memory use
+// 16-column chunks (mma3_ts16), so that each epilogue runs in two halves of
+// 16 columns and rewrites only columns it has already read.
 struct UpIn {
-  int64_t s;       // sample index (-1 past the list end)
+  int32_t s;       // sample index (-1 past the list end); act's 704 bytes per list position keep it in 32 bits
   int32_t r;
   float ws;
   float g[kOut];   // the upstream colour gradient, then (up_l3) g_z3
 };
 
 __device__ __forceinline__ void up_l1(UpIn& u, const int32_t* __restrict__ idx, int64_t j, int64_t n) {
-  u.s = j < n ? (idx ? (int64_t)__ldg(idx + j) : j) : -1;
+  u.s = j < n ? (idx ? __ldg(idx + j) : (int32_t)j) : -1;
 }
 __device__ __forceinline__ void up_l2(UpIn& u, const float* __restrict__ g_rgb, const float* __restrict__ w,
                                       const int32_t* __restrict__ ray_id) {
   if (u.s < 0) return;
   if (g_rgb) {
 #pragma unroll
-    for (int c = 0; c < kOut; ++c) u.g[c] = __ldg(g_rgb + 3 * u.s + c);
+    for (int c = 0; c < kOut; ++c) u.g[c] = __ldg(g_rgb + 3 * (int64_t)u.s + c);
   } else {
     u.ws = __ldg(w + u.s);
     u.r = __ldg(ray_id + u.s);
@@ -890,7 +990,7 @@ __device__ __forceinline__ void up_l3(UpIn& u, const float* __restrict__ g_rgb,
   if (u.s < 0) return;
   float y[kOut];
 #pragma unroll
-  for (int c = 0; c < kOut; ++c) y[c] = __ldg(rgb + 3 * u.s + c);
+  for (int c = 0; c < kOut; ++c) y[c] = __ldg(rgb + 3 * (int64_t)u.s + c);
   if (!g_rgb) {
 #pragma unroll
     for (int c = 0; c < kOut; ++c) u.g[c] = u.ws * __ldg(g_color + 3 * (int64_t)u.r + c);
@@ -910,7 +1010,7 @@ __device__ __forceinline__ bool bwd_wait(Side* fs, uint64_t* bar, uint32_t parit
 }
 
 template <class Op>
-__global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
+__global__ void __launch_bounds__(kThreads, 1) rgbnet_bwd_tc_kernel(
     const float* __restrict__ g_rgb, const float* __restrict__ g_color, const float* __restrict__ w,
     const float* __restrict__ rgb, const int32_t* __restrict__ ray_id, const int32_t* __restrict__ idx,
     int64_t n_cap, const int64_t* __restrict__ n_dev, const float* __restrict__ params,
@@ -932,9 +1032,11 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
     tc::mbar_init(&fs->bar_x, 1);
     tc::mbar_init(&fs->bar_d2, 1);
     tc::mbar_init(&fs->bar_gh, 1);
+    tc::mbar_init(&fs->bar_dw2a, 1);
     tc::mbar_init(&fs->bar_dw2, 1);
     tc::mbar_init(&fs->bar_gx, 1);
     tc::mbar_init(&fs->bar_fin, 1);
+    tc::mbar_init(&fs->g2a_full, 16);
     tc::mbar_init(&fs->g2_full, 16);
     tc::mbar_init(&fs->g1_full, 16);
     fs->abort = 0;
@@ -946,28 +1048,23 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
       tc::bulk_g2s(img + iX, img_g + (size_t)tile_of(0) * kImage + iX, 2 * kXBytes, &fs->bar_x);
     }
   }
-  UpIn cur, nxt;
-  if (compute) up_l1(cur, idx, tile_of(0) * kTile + row, n);
-  // scales: W2 and W1[:, 0:16] per matrix; G2 from the upstream bound, G1 from G2's
-  float m1 = 0.0f, m3 = 0.0f;
-#pragma unroll 4
-  for (int e = tid; e < kHid * 16; e += blockDim.x)
-    m1 = fmaxf(m1, fabsf(__ldg(params + kOffW1 + (e >> 4) * kIn + (e & 15))));
-  const float m2 = abs_max_part(params + kOffW2, kHid * kHid);
-  for (int o = tid; o < kHid; o += blockDim.x) {
-    float a = 0.0f;
+  float4* red = reinterpret_cast<float4*>(sm + bGh);   // block_max4 scratch (G is free until the first tile)
+  UpIn up;
+  if (compute && qw < 2) up_l1(up, idx, tile_of(0) * kTile + row, n);
+  // scales: W2 and W1[:, 0:16] per matrix; G2 from the upstream bound, G1 from G2's.
+  // gm: the largest upstream colour gradient over this CTA's own tiles (S2
+  // and S1 need only be uniform within the CTA: its partial gradient row
+  // carries its own scale).
+  W2Chunks w2;
+  W1Chunks16 w1;
+  w2.load(params);
+  w1.load(params);
+  if (compute && qw == 1) up_l2(up, g_rgb, w, ray_id);   // the first tile's rows
+  float m3 = 0.0f, gm = 0.0f;
+  if (tid < kHid) {
 #pragma unroll
-    for (int c = 0; c < kOut; ++c) a += fabsf(params[kOffW3 + c * kHid + o]);
-    m3 = fmaxf(m3, a);
+    for (int c = 0; c < kOut; ++c) m3 += fabsf(__ldg(params + kOffW3 + c * kHid + tid));
   }
-  const float mw1 = block_max(m1, fs->red);
-  const float mw2 = block_max(m2, fs->red);
-  const float mw3 = block_max(m3, fs->red);
-  const float sW1 = pow2_scale(mw1), sW2 = pow2_scale(mw2);
-  // Largest upstream colour gradient over this CTA's own tiles.  S2 and S1
-  // need only be uniform within the CTA: its partial gradient row carries
-  // its own scale.
-  float gm = 0.0f;
   {
     const int64_t cnt = nt * kTile;
     for (int64_t e0 = tid; e0 < cnt; e0 += 4 * (int64_t)blockDim.x) {
@@ -978,27 +1075,65 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
         const int64_t j = tile_of(e / kTile) * kTile + e % kTile;
         sv[u] = (e < cnt && j < n) ? (idx ? (int64_t)__ldg(idx + j) : j) : -1;
       }
+      float g[4][kOut];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        if (sv[u] < 0) continue;
-        float g[kOut];
-        upstream_rgb_grad(g_rgb, g_color, w, ray_id, sv[u], g);
-        gm = fmaxf(gm, fmaxf(fabsf(g[0]), fmaxf(fabsf(g[1]), fabsf(g[2]))));
+        g[u][0] = g[u][1] = g[u][2] = 0.0f;
+        if (sv[u] >= 0) upstream_rgb_grad(g_rgb, g_color, w, ray_id, sv[u], g[u]);
       }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) gm = fmaxf(gm, fmaxf(fabsf(g[u][0]), fmaxf(fabsf(g[u][1]), fabsf(g[u][2]))));
     }
   }
-  const float gmax = block_max(gm, fs->red);
+  if (compute && qw == 1) up_l3(up, g_rgb, g_color, rgb);
+  const float4 bm = block_max4(make_float4(w1.abs_max(), w2.abs_max(), m3, gm), red);
+  const float mw2 = bm.y, mw3 = bm.z, gmax = bm.w;
+  const float sW1 = pow2_scale(bm.x), sW2 = pow2_scale(mw2);
   // |g_z2[s]| <= max_o sum_c |W3[c][o]| * max_c |g_z3[s][c]| and g_z3 <= g_rgb / 4;
   // |g_h1[s]| <= 128 max|W2| max|g_z2[s]|.  S2 / S1: the scales of the largest bounds.
   const float w21 = mw2 * (float)kHid;
   const float S2 = pow2_scale(0.25f * gmax * mw3);
   const float S1 = pow2_scale(0.25f * gmax * mw3 * w21);
-  if (compute) up_l2(cur, g_rgb, w, ray_id);
   // W1[:, 0:16] split, hi and lo core matrices side by side in each 8-row
   // group, so that [hi | lo] is one 32-wide B operand of g_X = G1 W1[:, 0:16]
-  load_w1<Op, 16>(params, sm + bW1h, sm + bW1h + 256, kSboW1s, sW1);
-  load_w2<Op>(params, sm + bW2h, sm + bW2l, sW2);
-  if (compute) up_l3(cur, g_rgb, g_color, rgb);
+  w1.store<Op>(sm + bW1h, sm + bW1h + 256, kSboW1s, sW1);
+  w2.store<Op>(sm + bW2h, sm + bW2l, sW2);
+  // Upstream rows.  Column quarter 1's warps load the row's g_z3 of the next
+  // tile while they wait for this tile's g_h1, and leave it with its scales in
+  // shared memory for all: gradient scales of the row for g_h1 (sG2) and g_X
+  // (sG1), the weight-gradient products take the CTA-wide S2, S1 instead.
+  float db3acc[kOut] = {0.0f, 0.0f, 0.0f}, rowg[kOut], rowr;
+  uint32_t rowe;
+  bool rowtiny;
+  auto row_scales = [&]() {   // from `up` (after up_l3)
+#pragma unroll
+    for (int c = 0; c < kOut; ++c) {
+      rowg[c] = up.s >= 0 ? up.g[c] : 0.0f;
+      db3acc[c] += rowg[c];
+    }
+    const float b2s = mw3 * fmaxf(fabsf(rowg[0]), fmaxf(fabsf(rowg[1]), fabsf(rowg[2])));
+    const float sG2 = b2s > 0.0f ? fmaxf(pow2_scale(b2s), S2) : S2;
+    const float sG1 = b2s > 0.0f ? fmaxf(pow2_scale(b2s * w21), S1) : S1;
+    rowr = pow2_rcp(sG2);
+    rowe = (__float_as_uint(sG2) >> 23) | ((__float_as_uint(sG1) >> 23) << 8);
+    rowtiny = S2 * rowr < Op::kMinFactor;
+#pragma unroll
+    for (int c = 0; c < kOut; ++c) rowg[c] *= sG2;
+  };
+  auto row_store = [&](int64_t k) {   // rows of tile k
+    float* q = reinterpret_cast<float*>(&fs->smp[row >> 1][0]) + (row & 1);
+    q[0] = rowg[0];
+    q[2] = rowg[1];
+    q[4] = rowg[2];
+    q[6] = rowr;
+    fs->sc[k & 1][row] = (uint16_t)rowe;
+    const bool any = __any_sync(0xffffffffu, rowtiny);
+    if (lane == 0) fs->tiny[warp & 3] = any ? 1u : 0u;
+  };
+  if (compute && qw == 1) {
+    row_scales();
+    row_store(0);
+  }
   tc::fence_proxy_async_smem();
   tc::fence_before_sync();
   __syncthreads();
@@ -1010,8 +1145,17 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
   const uint32_t sHh = tc::smem_u32(img + iHh), sHl = tc::smem_u32(img + iHl);
   const uint32_t sGh = tc::smem_u32(sm + bGh), sGl = tc::smem_u32(sm + bGl);
   float vmax = 0.0f;   // largest magnitude split (range check)
-  // per-thread partial sums of dW3, db2 (hidden unit oh) and db3 (tile row)
-  float dW3acc[kOut] = {0.0f, 0.0f, 0.0f}, db2acc = 0.0f, db3acc[kOut] = {0.0f, 0.0f, 0.0f};
+  // H1 terms of tile k's rows 32 q + 16 half .. + 15 (q < 4; one thread)
+  auto copy_h_half = [&](int64_t k, int half) {
+    const uint8_t* src = img_g + (size_t)tile_of(k) * kImage;
+#pragma unroll
+    for (uint32_t q = 0; q < 8; ++q) {
+      const uint32_t off = iHh + (q >> 2) * kHBytes + (4 * (q & 3) + 2 * (uint32_t)half) * kSboH;
+      tc::bulk_g2s(img + off, src + off, 2 * kSboH, &fs->bar_h);
+    }
+  };
+  // per-thread partial sums of dW3 and db2 (hidden unit oh; even and odd rows)
+  f32x2 dW3acc[kOut] = {0ull, 0ull, 0ull}, db2acc = 0ull;
   if (warp == 16) {
     // ------------------------------------------------------------ MMA warp
     // lane 0 polls (the outcome of a wait is the warp's); the elected thread issues
@@ -1020,8 +1164,9 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
       if (lane == 0) r = bwd_wait(fs, bar, parity) ? 1 : 0;
       return __shfl_sync(0xffffffffu, r, 0) != 0;
     };
-    bool inflight_x = nt > 0;   // elected thread: an X copy not yet seen landed
-    uint32_t ph_h = 0, ph_x = 0, ph_gx = 0, ph_g2 = 0, ph_g1 = 0;
+    // elected thread: copies not yet seen landed
+    bool inflight_x = nt > 0, inflight_h = nt > 0;
+    uint32_t ph_h = 0, ph_x = 0, ph_gx = 0, ph_g2a = 0, ph_g2 = 0, ph_g1 = 0, ph_dw2a = 0;
     auto load_x = [&](int64_t k) {
       tc::mbar_arrive_expect_tx(&fs->bar_x, 2 * kXBytes);
       tc::bulk_g2s(img + iX, img_g + (size_t)tile_of(k) * kImage + iX, 2 * kXBytes, &fs->bar_x);
@@ -1029,20 +1174,22 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
     };
     // D2^T = W2 H1^T of the tile whose H1 terms have landed (TMEM lane =
     // hidden unit, column = tile row); after a failed wait only the commit
-    auto d2 = [&](bool h_ok) {
-      if (h_ok) {
-        mma3<kHid / 16, Op::kWeightLo, true>(tmem + cTmp, sW2h, sW2l, 256, 128, kSboH, sHh, sHl, 256, 128, kSboH,
-                                             Op::idesc(128, kTile, 0, 0), false);
-      }
-      tc::mma_commit(&fs->bar_d2);
-    };
-    if (nt > 0) {
+    auto wait_h_d2 = [&]() {
       const bool h_ok = wait0(&fs->bar_h, ph_h);
-      ph_h ^= 1;
+      if (h_ok) {
+        inflight_h = false;
+        ph_h ^= 1;
+      }
       tc::fence_after_sync();
-      if (tc::elect_one()) d2(h_ok);
+      if (tc::elect_one()) {
+        if (h_ok)
+          mma3<kHid / 16, Op::kWeightLo, true>(tmem + cTmp, sW2h, sW2l, 256, 128, kSboH, sHh, sHl, 256, 128, kSboH,
+                                               Op::idesc(128, kTile, 0, 0), false);
+        tc::mma_commit(&fs->bar_d2);
+      }
       __syncwarp();
-    }
+    };
+    if (nt > 0) wait_h_d2();
     for (int64_t k = 0; k < nt; ++k) {
       const bool has_next = k + 1 < nt;
       // X(k): the buffer is free once g_X and dW1 of tile k - 1 are done
@@ -1051,14 +1198,42 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
         __syncwarp();
         ph_gx ^= 1;
       }
-      // dW2 += G2^T H1 (A from tensor memory), then g_h1 = G2 W2 (A MN-major)
+      // a later tile's image starts its way into L2, so that its copies into
+      // shared memory do not wait for DRAM
+      if (k + 2 < nt && tc::elect_one()) tc::bulk_prefetch_l2(img_g + (size_t)tile_of(k + 2) * kImage, kImage);
+      __syncwarp();
+      // dW2 += G2^T H1 (A from tensor memory) over the rows 32 q .. 32 q + 15,
+      // while the compute warps form G2 of the others; then those rows' H1
+      // terms of the next tile
+      const bool g2a = wait0(&fs->g2a_full, ph_g2a);
+      ph_g2a ^= 1;
+      tc::fence_after_sync();
+      if (tc::elect_one()) {
+        if (g2a)
+          mma3_ts16<kTile / 32, 2>(tmem + cDW2, tmem + cTmp, sHh, sHl, 2 * kSboH, kSboH, 128,
+                                   Op::idesc(128, kHid, 0, 1), k > 0);
+        tc::mma_commit(&fs->bar_dw2a);
+      }
+      __syncwarp();
+      if (has_next) {
+        if (wait0(&fs->bar_dw2a, ph_dw2a)) {
+          inflight_h = true;
+          if (tc::elect_one()) {
+            tc::mbar_arrive_expect_tx(&fs->bar_h, 2 * kHBytes);   // both halves
+            copy_h_half(k + 1, 0);
+          }
+          __syncwarp();
+        }
+        ph_dw2a ^= 1;
+      }
+      // the other rows' dW2, then g_h1 = G2 W2 (A MN-major)
       const bool g2 = wait0(&fs->g2_full, ph_g2);
       ph_g2 ^= 1;
       tc::fence_after_sync();
       if (tc::elect_one()) {
         if (g2)
-          mma3_ts16<kTile / 16>(tmem + cDW2, tmem + cTmp, sHh, sHl, 2 * kSboH, kSboH, 128,
-                                Op::idesc(128, kHid, 0, 1), k > 0);
+          mma3_ts16<kTile / 32, 2>(tmem + cDW2, tmem + cTmp + 16u, sHh + 2 * kSboH, sHl + 2 * kSboH, 2 * kSboH, kSboH,
+                                   128, Op::idesc(128, kHid, 0, 1), true);
         tc::mma_commit(&fs->bar_dw2);
         if (g2)
           mma3<kHid / 16, true, Op::kWeightLo>(tmem + cGH, sGh, sGl, 2 * kSboH, kSboH, 128, sW2h, sW2l, 2 * kSboH,
@@ -1066,15 +1241,8 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
         tc::mma_commit(&fs->bar_gh);
       }
       __syncwarp();
-      // the next tile's D2^T once its H1 has landed (compute thread 0 copies
-      // it in when dW2 has read this one's); it needs no G1 of this tile
-      if (has_next) {
-        const bool h_ok = wait0(&fs->bar_h, ph_h);
-        ph_h ^= 1;
-        tc::fence_after_sync();
-        if (tc::elect_one()) d2(h_ok);
-        __syncwarp();
-      }
+      // the next tile's D2^T once its H1 has landed; it needs no G1 of this tile
+      if (has_next) wait_h_d2();
       // once G1 and X are in: g_X = G1 W1[:, 0:16] (A from tensor memory) and
       // dW1|db1 += G1^T X
       const bool g1 = wait0(&fs->g1_full, ph_g1);
@@ -1082,9 +1250,9 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
       tc::fence_after_sync();
       if (tc::elect_one()) {
         const bool x_ok = g1 && bwd_wait(fs, &fs->bar_x, ph_x);
-        ph_x ^= 1;
         if (x_ok) {
           inflight_x = false;
+          ph_x ^= 1;
           {   // per K step: G1h [W1h | W1l] (N = 32: hi*hi in columns 0-15, hi*lo in 16-31), G1l W1h
             const uint32_t id32 = Op::idesc(128, 32, 0, 1), id16 = Op::idesc(128, 16, 0, 1);
             uint64_t db = tc::smem_desc(sW1h, kSboW1s, 128);
@@ -1124,20 +1292,25 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
         set_status(DVGO_ERR_TIMEOUT);
       }
       if (inflight_x) tc::mbar_wait(&fs->bar_x, ph_x, kSpin);
+      if (inflight_h) tc::mbar_wait(&fs->bar_h, ph_h, kSpin);
     }
     __syncwarp();
   } else {
     // -------------------------------------------------------- compute warps
     const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const float inv2 = 1.0f / (kSH * sW2);           // D2 -> z2 - b2
+    const float rinv2 = kSH * sW2;   // D2 = kSH sW2 (z2 - b2): z2 and h2 are kept at this scale
     // this thread's hidden unit in the transposed layer-2 products (TMEM lane)
     const int oh = (warp & 3) * 32 + lane;
     const float b2o = Op::param(__ldg(params + kOffB2 + oh)), w3o0 = Op::param(__ldg(params + kOffW3 + oh)),
                 w3o1 = Op::param(__ldg(params + kOffW3 + kHid + oh)),
                 w3o2 = Op::param(__ldg(params + kOffW3 + 2 * kHid + oh));
     uint32_t ph_h = 0, ph_d2 = 0, ph_gh = 0, ph_gx = 0, ph_dw2 = 0;
-    bool inflight_h = tid == 0 && nt > 0;   // thread 0: an H1 copy not yet seen landed
-    int64_t prev_s = -1;       // the previous tile's row: its g_X is stored one tile later
+    const f32x2 b2x = pack2(b2o * rinv2, b2o * rinv2), w0x = pack2(w3o0, w3o0),
+                w1x = pack2(w3o1, w3o1), w2x = pack2(w3o2, w3o2), S2x = pack2(S2, S2);
+    const float rW2 = pow2_rcp(sW2), rW1 = pow2_rcp(sW1);
+    // this row's sample in the current and the previous tile (quarter 0: its
+    // g_X is stored one tile later), and in the next one (quarters 0 and 1)
+    int32_t s_cur = qw < 2 ? up.s : -1, prev_s = -1;
     float prev_invX = 0.0f;
     // g_X = G1 W1[:, 0:16] of the previous tile (lane quarter qw == 0) -> g_k0
     auto store_gx = [&]() {
@@ -1145,7 +1318,7 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
       tc::tmem_ld16(lane_base + cGX, ga);
       tc::tmem_ld16(lane_base + cGX + 16, gb);
       if (prev_s >= 0) {
-        float4* dst = reinterpret_cast<float4*>(g_k0 + prev_s * kFeat);
+        float4* dst = reinterpret_cast<float4*>(g_k0 + (int64_t)prev_s * kFeat);
 #pragma unroll
         for (int q = 0; q < 3; ++q)
           dst[q] = make_float4((ga[4 * q] + gb[4 * q]) * prev_invX, (ga[4 * q + 1] + gb[4 * q + 1]) * prev_invX,
@@ -1153,83 +1326,60 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
                                (ga[4 * q + 3] + gb[4 * q + 3]) * prev_invX);
       }
     };
-    for (int64_t k = 0; k < nt; ++k) {
-      const bool valid = cur.s >= 0;
-      const int64_t s = cur.s;
-      up_l1(nxt, idx, tile_of(k + 1) * kTile + row, n);
-      // this tile's H1 terms (for the relu mask)
-      if (bwd_wait(fs, &fs->bar_h, ph_h)) inflight_h = false;
+    // relu mask of layer 1 on this quarter's columns of a tile whose H1 terms
+    // have landed (H1 > 0 <=> hi > 0): column 2 i + b of the quarter in bit i + 16 b
+    auto relu_mask = [&]() -> uint32_t {
+      bwd_wait(fs, &fs->bar_h, ph_h);
       ph_h ^= 1;
-      // g_z3 of this row's sample and its gradient scales (for g_h1 and g_X);
-      // the weight-gradient products take the CTA-wide S2, S1 instead
-      float fG1, invX, r1;
-      {
-        float gz3[kOut] = {0.0f, 0.0f, 0.0f};
-        if (valid) {
-#pragma unroll
-          for (int c = 0; c < kOut; ++c) gz3[c] = cur.g[c];
-        }
-        const float b2s = mw3 * fmaxf(fabsf(gz3[0]), fmaxf(fabsf(gz3[1]), fabsf(gz3[2])));
-        const float sG2 = b2s > 0.0f ? fmaxf(pow2_scale(b2s), S2) : S2;
-        const float sG1 = b2s > 0.0f ? fmaxf(pow2_scale(b2s * w21), S1) : S1;
-        fG1 = sG1 / (sG2 * sW2);             // (sG2 G2)(sW2 W2) -> sG1 g_h1
-        invX = 1.0f / (sG1 * sW1);           // g_X
-        r1 = S1 / sG1;                       // G1 terms -> the dW1 copy
-        if (qw == 0) {
-          fs->smp[row] = make_float4(gz3[0], gz3[1], gz3[2], sG2);
-#pragma unroll
-          for (int c = 0; c < kOut; ++c) db3acc[c] += gz3[c];
-        }
-      }
-      // relu mask of layer 1 on this quarter's columns (H1 > 0 <=> hi > 0)
-      uint32_t m1b = 0u;
+      uint32_t m = 0u;
 #pragma unroll
       for (int k8 = 0; k8 < 32; k8 += 8) {
         const uint4 q = *reinterpret_cast<const uint4*>(img + iHh + tc::cm_off(row, 32 * qw + k8, kSboH));
         const uint32_t wd[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int kq = k8 + 2 * i;
-          if ((int16_t)(wd[i] & 0xffffu) > 0) m1b |= 1u << kq;
-          if ((int16_t)(wd[i] >> 16) > 0) m1b |= 1u << (kq + 1);
-        }
+        for (int i = 0; i < 4; ++i) m |= Op::positive(wd[i]) & (0x00010001u << (k8 / 2 + i));
       }
-      up_l2(nxt, g_rgb, w, ray_id);
-      tc::named_sync(1, 512);   // every row's g_z3 and scale are in fs->smp
+      return m;
+    };
+    uint32_t m1b = 0u, m1b_next = nt > 0 ? relu_mask() : 0u;
+    for (int64_t k = 0; k < nt; ++k) {
+      if (qw < 2) up_l1(up, idx, tile_of(k + 1) * kTile + row, n);
+      m1b = m1b_next;
+      tc::named_sync(1, 512);   // every row's g_z3 and scales are in shared memory
       bwd_wait(fs, &fs->bar_d2, ph_d2);
       ph_d2 ^= 1;
       tc::fence_after_sync();
       // Hidden unit oh over the tile rows 32 qw .. 32 qw + 31 (two halves of
-      // 16): G2 = (W3^T g_z3) * (z2 > 0), and the sums over rows dW3 +=
-      // g_z3 h2^T, db2 += G2 in registers.  G2 goes out twice: at the
-      // CTA-wide scale S2 into tensor memory over the half's own D2 columns
-      // (lane = unit, K = row: the A operand of dW2), and at each row's own
-      // scale sG2 into shared memory as [unit][row] core matrices (the
-      // MN-major A operand of g_h1).
+      // 16, two rows per packed instruction): G2 = (W3^T g_z3) * (z2 > 0), and
+      // the sums over rows dW3 += g_z3 h2^T, db2 += G2 in registers.  G2 is
+      // formed and split at each row's own scale sG2 and goes out twice: as
+      // [unit][row] core matrices into shared memory (the MN-major A operand
+      // of g_h1), and with its terms times S2 / sG2 (the CTA-wide scale S2)
+      // into tensor memory over the half's own D2 columns (lane = unit, K =
+      // row: the A operand of dW2).  A factor too small for the term format
+      // (a row 2^-24 below the CTA's largest) takes a split of its own.
+      const bool tiny = fs->tiny[qw] != 0u;
 #pragma unroll 1
       for (int h = 0; h < 2; ++h) {
         const int r0 = 32 * qw + 16 * h;
         float v[16];
         tc::tmem_ld16(lane_base + cTmp + r0, v);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const float4 q = fs->smp[r0 + i];
-          const float z2 = fmaf(v[i], inv2, b2o);
-          const float gs = fmaf(w3o2, q.z, fmaf(w3o1, q.y, w3o0 * q.x));
-          const float g = z2 > 0.0f ? gs : 0.0f;
-          const float hh = fmaxf(z2, 0.0f);
-          db2acc += g;
-          dW3acc[0] = fmaf(q.x, hh, dW3acc[0]);
-          dW3acc[1] = fmaf(q.y, hh, dW3acc[1]);
-          dW3acc[2] = fmaf(q.z, hh, dW3acc[2]);
-          v[i] = g;
-        }
         uint32_t hl[16];
-        split16<Op>(v, S2, hl, vmax);
-        tc::tmem_st16(lane_base + cTmp + r0, hl);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] *= fs->smp[r0 + i].w;
-        split16<Op>(v, 1.0f, hl, vmax);
+        for (int c = 0; c < 8; ++c) {
+          const float4 qa = fs->smp[(r0 >> 1) + c][0], qb = fs->smp[(r0 >> 1) + c][1];
+          const f32x2 gx = pack2(qa.x, qa.y), gy = pack2(qa.z, qa.w), gz = pack2(qb.x, qb.y),
+                      rs = pack2(qb.z, qb.w);
+          const float2 z2 = unpack2(add2(pack2(v[2 * c], v[2 * c + 1]), b2x));
+          const float2 gs = unpack2(fma2(w2x, gz, fma2(w1x, gy, mul2(w0x, gx))));
+          const f32x2 g = pack2(z2.x > 0.0f ? gs.x : 0.0f, z2.y > 0.0f ? gs.y : 0.0f);
+          const f32x2 hr = mul2(pack2(fmaxf(z2.x, 0.0f), fmaxf(z2.y, 0.0f)), rs);
+          db2acc = fma2(g, rs, db2acc);
+          dW3acc[0] = fma2(gx, hr, dW3acc[0]);
+          dW3acc[1] = fma2(gy, hr, dW3acc[1]);
+          dW3acc[2] = fma2(gz, hr, dW3acc[2]);
+          hl[c] = split_pair<Op>(g, hl[8 + c], vmax);
+        }
         // the previous tile's g_X and dW1 (readers of G's shared memory, X and
         // the g_X columns) are done
         if (h == 0 && k > 0) {
@@ -1238,37 +1388,66 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
           tc::fence_after_sync();
         }
         st_terms16<Op, false>(sm + bGh, sm + bGl, oh, r0, hl, 1.0f);
-      }
-      if (k > 0 && qw == 0) store_gx();
-      tc::tmem_wait_st();
-      tc::fence_proxy_async_smem();
-      tc::fence_before_sync();
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&fs->g2_full);
-      up_l3(nxt, g_rgb, g_color, rgb);
-      // the next tile's H1 terms, once dW2 has read this tile's
-      if (tid == 0 && k + 1 < nt) {
-        if (bwd_wait(fs, &fs->bar_dw2, ph_dw2)) {
-          tc::mbar_arrive_expect_tx(&fs->bar_h, 2 * kHBytes);
-          tc::bulk_g2s(img + iHh, img_g + (size_t)tile_of(k + 1) * kImage + iHh, 2 * kHBytes, &fs->bar_h);
-          inflight_h = true;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const float2 q = reinterpret_cast<const float2*>(&fs->smp[(r0 >> 1) + c][1])[1];
+          const f32x2 f2 = mul2(S2x, pack2(q.x, q.y));
+          if (tiny) {
+            hl[c] = split_pair<Op>(mul2(Op::join2(hl[c], hl[8 + c]), f2), hl[8 + c], vmax);
+          } else {
+            const float2 f = unpack2(f2);
+            const uint32_t fac = Op::pack(f.x, f.y);
+            hl[c] = Op::mul2v(hl[c], fac);
+            hl[8 + c] = Op::mul2v(hl[8 + c], fac);
+          }
         }
+        tc::tmem_st16(lane_base + cTmp + r0, hl);
+        if (h == 1 && k > 0 && qw == 0) store_gx();
+        tc::tmem_wait_st();
+        tc::fence_proxy_async_smem();
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(h == 0 ? &fs->g2a_full : &fs->g2_full);
+      }
+      // the next tile's H1 terms of the second half of the rows, once dW2 has
+      // read this tile's (the first half's copy runs already)
+      if (tid == 0 && k + 1 < nt) {
+        if (bwd_wait(fs, &fs->bar_dw2, ph_dw2)) copy_h_half(k + 1, 1);
         ph_dw2 ^= 1;
       }
+      __syncwarp();
+      // the next tile's upstream rows, while g_h1 runs
+      if (qw == 1 && k + 1 < nt) {
+        up_l2(up, g_rgb, w, ray_id);
+        up_l3(up, g_rgb, g_color, rgb);
+        row_scales();
+      }
+      if (k + 1 < nt) m1b_next = relu_mask();
       bwd_wait(fs, &fs->bar_gh, ph_gh);
       ph_gh ^= 1;
       tc::fence_after_sync();
+      // every warp has passed its G2 epilogue (bar_gh follows g2_full): the
+      // rows of this tile have been read
+      if (qw == 1 && k + 1 < nt) row_store(k + 1);
       // G1 = g_h1 * (H1 > 0): at S1 in shared memory (dW1), at sG1 in tensor
       // memory (g_X), in two halves of 16 hidden units
+      const uint32_t e = fs->sc[k & 1][row];
+      const float sG1 = __uint_as_float((e >> 8) << 23), rG1 = pow2_rcp(sG1);
+      const float fG1 = sG1 * pow2_rcp(__uint_as_float((e & 0xffu) << 23)) * rW2;   // (sG2 G2)(sW2 W2) -> sG1 g_h1
+      const float r1 = S1 * rG1;                                                    // G1 terms -> the dW1 copy
+      const f32x2 fG1x = pack2(fG1, fG1);
 #pragma unroll 1
       for (int h = 0; h < 2; ++h) {
         const int c0 = 32 * qw + 16 * h;
         float v[16];
         tc::tmem_ld16(lane_base + cGH + c0, v);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = ((m1b >> (16 * h + i)) & 1u) ? v[i] : 0.0f;
         uint32_t hl[16];
-        split16<Op>(v, fG1, hl, vmax);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const f32x2 g = pack2((m1b >> c) & 1u ? v[2 * c] : 0.0f, (m1b >> (16 + c)) & 1u ? v[2 * c + 1] : 0.0f);
+          hl[c] = split_pair<Op>(mul2(g, fG1x), hl[8 + c], vmax);
+        }
+        m1b >>= 8;
         tc::tmem_st16(lane_base + cGH + c0, hl);
         st_terms16<Op>(sm + bGh, sm + bGl, row, c0, hl, r1);
       }
@@ -1277,9 +1456,9 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&fs->g1_full);
-      prev_s = valid ? s : -1;
-      prev_invX = invX;
-      cur = nxt;
+      prev_s = s_cur;
+      prev_invX = rG1 * rW1;
+      s_cur = up.s;
     }
     // the last tile's g_X
     if (nt > 0) {
@@ -1287,8 +1466,6 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
       tc::fence_after_sync();
       if (qw == 0) store_gx();
     }
-    // a copy issued but never seen landed (only after a failed wait) lands before exit
-    if (inflight_h) tc::mbar_wait(&fs->bar_h, ph_h, kSpin);
   }
   tc::fence_before_sync();
   __syncthreads();
@@ -1303,10 +1480,14 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
   float* pr3 = pr + 16 * 4 * 32;                             // [4 lane quarters][3]
   if (compute) {
 #pragma unroll
-    for (int c = 0; c < kOut; ++c) pr[(warp * 4 + c) * 32 + lane] = dW3acc[c];
-    pr[(warp * 4 + 3) * 32 + lane] = db2acc;
+    for (int c = 0; c < kOut; ++c) {
+      const float2 f = unpack2(dW3acc[c]);
+      pr[(warp * 4 + c) * 32 + lane] = (f.x + f.y) * pow2_rcp(kSH * sW2);
+    }
+    const float2 f = unpack2(db2acc);
+    pr[(warp * 4 + 3) * 32 + lane] = f.x + f.y;
   }
-  if (compute && qw == 0) {
+  if (compute && qw == 1) {
 #pragma unroll
     for (int c = 0; c < kOut; ++c) {
       float v = db3acc[c];
@@ -1318,7 +1499,7 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  float* P = part + (size_t)blockIdx.x * kNumParams;
+  float* P = part + (size_t)blockIdx.x * kPartRow;
   const bool has_tiles = (int64_t)blockIdx.x < ntiles;
   if (has_tiles && compute && qw == 0) {   // warp l: W3[:, 32 l + lane] and b2[32 l + lane] over the 4 row quarters
 #pragma unroll
@@ -1328,47 +1509,48 @@ __global__ void __launch_bounds__(544, 1) rgbnet_bwd_tc_kernel(
       P[(c < kOut ? kOffW3 + c * kHid : kOffB2) + 32 * warp + lane] = v;
     }
   }
-  if (has_tiles && tid < kOut) P[kOffB3 + tid] = ((pr3[tid] + pr3[kOut + tid]) + pr3[2 * kOut + tid]) + pr3[3 * kOut + tid];
+  if (has_tiles && tid < kOut)
+    part[(size_t)kNumSMs * kPartRow + blockIdx.x * kOut + tid] =
+        ((pr3[tid] + pr3[kOut + tid]) + pr3[2 * kOut + tid]) + pr3[3 * kOut + tid];
   if (has_tiles && compute) {
     const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    // dW2 / dW1 rows (TMEM lane = output neuron) through a per-warp 32 x 33
-    // shared-memory transpose, so that each store covers 32 consecutive
-    // parameters of one row
-    float* tp = reinterpret_cast<float*>(sm + bImg) + warp * 32 * 33;
     const float u2 = ok ? 1.0f / (S2 * kSH) : 0.0f, u1 = ok ? 1.0f / (S1 * kSX) : 0.0f;
     const int o0 = (warp & 3) * 32;
-    // columns col (plus columns col2, when given) of this warp's 32 lanes
-    auto flush32 = [&](uint32_t col, float scale, int base, int stride, uint32_t col2 = 0) {
-      float v[32];
-      tc::tmem_ld32(lane_base + col, v);
-      if (col2) {
-        float v2[32];
-        tc::tmem_ld32(lane_base + col2, v2);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] += v2[i];
-      }
-#pragma unroll
-      for (int i = 0; i < 32; ++i) tp[lane * 33 + i] = v[i] * scale;
-      __syncwarp();
-      for (int r = 0; r < 32; ++r) P[base + (o0 + r) * stride + lane] = tp[r * 33 + lane];
-      __syncwarp();
-    };
-    flush32(cDW2 + 32 * qw, u2, kOffW2 + 32 * qw, kHid);
-    // dW1 | db1: the sum of the hi*hi + lo*hi columns and the hi*lo columns
-    if (qw == 0) {
-      flush32(cDW1, u1, kOffW1, kIn, cDW1 + kK1);              // W1[:, 0:32]
-    } else if (qw == 1) {
+    // dW1 | db1: the sum of the hi*hi + lo*hi columns and the hi*lo columns;
+    // ten of the 40 columns per quarter, into rows of 39 and the bias after
+    // them, as they lie in the parameter vector (G's lo buffer is free)
+    float* raw1 = reinterpret_cast<float*>(sm + bGl);
+    {
       float v[16], v2[16];
-      tc::tmem_ld16(lane_base + cDW1 + 32, v);                  // W1[:, 32:39] and b1 (column 39)
-      tc::tmem_ld16(lane_base + cDW1 + kK1 + 32, v2);
+      tc::tmem_ld16(lane_base + cDW1 + 10 * qw, v);
+      tc::tmem_ld16(lane_base + cDW1 + kK1 + 10 * qw, v2);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) tp[lane * 33 + i] = (v[i] + v2[i]) * u1;
-      __syncwarp();
-      for (int r = 0; r < 32; ++r) {
-        if (lane < kIn - 32) P[kOffW1 + (o0 + r) * kIn + 32 + lane] = tp[r * 33 + lane];
-        else if (lane == kIn - 32) P[kOffB1 + o0 + r] = tp[r * 33 + lane];
+      for (int i = 0; i < 10; ++i) {
+        const int k = 10 * qw + i;
+        raw1[k < kIn ? (o0 + lane) * kIn + k : kHid * kIn + o0 + lane] = (v[i] + v2[i]) * u1;
       }
     }
+    // dW2 (TMEM lane = output neuron): the warp's 32 x 32 block through a
+    // 36-float-stride transpose, so that each store covers four 128-byte rows
+    float* tp = reinterpret_cast<float*>(sm + bImg) + warp * 32 * 36;
+    {
+      float v[32];
+      tc::tmem_ld32(lane_base + cDW2 + 32 * qw, v);
+#pragma unroll
+      for (int i = 0; i < 32; i += 4)
+        *reinterpret_cast<float4*>(tp + lane * 36 + i) =
+            make_float4(v[i] * u2, v[i + 1] * u2, v[i + 2] * u2, v[i + 3] * u2);
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < 32; r += 4) {
+        const int rr = r + (lane >> 3), cc = 4 * (lane & 7);
+        *reinterpret_cast<float4*>(P + kOffW2 + (o0 + rr) * kHid + 32 * qw + cc) =
+            *reinterpret_cast<const float4*>(tp + rr * 36 + cc);
+      }
+    }
+    tc::named_sync(1, 512);   // raw1 is complete
+    for (int e = tid; e < (kHid * kIn + kHid) / 4; e += 512)
+      *reinterpret_cast<float4*>(P + kOffW1 + 4 * e) = reinterpret_cast<const float4*>(raw1)[e];
   }
   tc::fence_before_sync();
   __syncthreads();
@@ -1391,7 +1573,8 @@ __global__ void __launch_bounds__(256) partials_reduce_kernel(const float* __res
   float a = 0.0f;
   if (p < kNumParams) {
 #pragma unroll 8
-    for (int b = b0; b < b1; ++b) a += __ldg(part + (size_t)b * kNumParams + p);
+    for (int b = b0; b < b1; ++b) a += __ldg(p < kPartRow ? part + (size_t)b * kPartRow + p
+                                                          : part + (size_t)kNumSMs * kPartRow + b * kOut + p - kPartRow);
   }
   acc[grp][j] = a;
   __syncthreads();
@@ -1408,7 +1591,8 @@ __global__ void __launch_bounds__(256) partials_reduce_kernel(const float* __res
 using namespace dvgo;
 
 // act layout: [256 reserved bytes | one 90112-byte image per 128-position tile |
-// kNumSMs partial gradient rows of kNumParams floats]
+// kNumSMs partial gradient rows of kPartRow floats (a multiple of 32, so that
+// rows start on 128-byte boundaries) | kNumSMs partial db3 of 3 floats]
 static int64_t act_images_end(int64_t n_cap) {
   return (int64_t)kActHeader + (n_cap + kTile - 1) / kTile * (int64_t)kImage;
 }
@@ -1428,7 +1612,7 @@ static int rgbnet_fwd_tc(const float* k0, const float* rays_d, const int32_t* ra
     attr = true;
   }
   const int grid = (int)std::min<int64_t>((n_cap + kTile - 1) / kTile, kNumSMs);
-  rgbnet_fwd_tc_kernel<Op><<<grid, 544, smem, st>>>(k0, rays_d, ray_id, idx, n_cap, n_dev, params, rgb,
+  rgbnet_fwd_tc_kernel<Op><<<grid, kThreads, smem, st>>>(k0, rays_d, ray_id, idx, n_cap, n_dev, params, rgb,
                                                     reinterpret_cast<uint8_t*>(act));
   return launch_status();
 }
@@ -1445,7 +1629,7 @@ static int rgbnet_bwd_tc(const float* g_rgb, const float* g_color, const float* 
   }
   const int grid = (int)std::min<int64_t>((n_cap + kTile - 1) / kTile, kNumSMs);
   float* part = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(act) + act_images_end(n_cap));
-  rgbnet_bwd_tc_kernel<Op><<<grid, 544, smem, st>>>(g_rgb, g_color, w, rgb, ray_id, idx, n_cap, n_dev,
+  rgbnet_bwd_tc_kernel<Op><<<grid, kThreads, smem, st>>>(g_rgb, g_color, w, rgb, ray_id, idx, n_cap, n_dev,
                                                     params, reinterpret_cast<const uint8_t*>(act), part,
                                                     g_k0);
   partials_reduce_kernel<<<(kNumParams + 31) / 32, 256, 0, st>>>(part, grid, n_cap, n_dev, g_params);

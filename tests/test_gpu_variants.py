@@ -1,0 +1,123 @@
+"""Kernel variants at the sizes where they can go wrong: edges of tiles and
+chunks, remainders, operands off their fast path's alignment."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2206_05085_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    from paper_2206_05085_gb300 import build
+    build.build()
+    from paper_2206_05085_gb300 import _lib
+    return _lib
+
+
+def _select_ref(q, off, n_draw):
+    """The header's rule, one candidate at a time in FP32."""
+    sel = np.full((len(off) - 1, n_draw), -1, np.int32)
+    cnt = np.zeros(len(off) - 1, np.int32)
+    u = ((np.arange(n_draw, dtype=np.float32) + np.float32(0.5)) / np.float32(n_draw)).astype(np.float32)
+    for r in range(len(off) - 1):
+        x = q[off[r]:off[r + 1]]
+        if len(x) == 0:
+            continue
+        j, cdf, out = 0, x[0], []
+        for k in range(n_draw):
+            while j < len(x) - 1 and not (u[k] < cdf):
+                j += 1
+                cdf = np.float32(cdf + x[j])
+            if not out or out[-1] != j:
+                out.append(j)
+        sel[r, :len(out)] = out
+        cnt[r] = len(out)
+    return sel, cnt
+
+
+@pytest.mark.parametrize("n_draw", [1, 7, 64, 130])
+def test_select_against_sequential_rule(L, n_draw):
+    rng = np.random.default_rng(3)
+    lens = [0, 1, 2, 3, 31, 32, 33, 127, 128, 129, 255, 256, 257, 0, 512, 5, 300]
+    rows = []
+    for i, n in enumerate(lens):
+        x = rng.random(n).astype(np.float32) ** 4
+        if n:
+            x /= np.float32(max(x.sum(), 1e-6))
+        if n > 4 and i % 4 == 0:
+            x[n // 2] = np.nan            # the CDF is NaN from here: nothing exceeds it
+        if n > 4 and i % 4 == 1:
+            x[1::3] *= -1                 # a CDF that falls again
+        if n > 4 and i % 4 == 2:
+            x[n // 3] = np.inf
+        rows.append(x)
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    q = np.concatenate(rows)
+    with np.errstate(invalid="ignore"):
+        ref_sel, ref_n = _select_ref(q, off, n_draw)
+    R = len(lens)
+    sel = torch.full((R * n_draw,), 7, dtype=torch.int32, device="cuda")
+    n_sel = torch.full((R,), 7, dtype=torch.int32, device="cuda")
+    L.proposal_select(torch.from_numpy(q).cuda(), torch.from_numpy(off).cuda(), R, n_draw, sel, n_sel)
+    assert np.array_equal(n_sel.cpu().numpy(), ref_n)
+    assert np.array_equal(sel.cpu().numpy().reshape(R, n_draw), ref_sel)
+
+
+@pytest.mark.parametrize("precision", ["f32tc", "bf16"])
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 152 * 128 + 1])
+def test_rgbnet_parameters_off_alignment(L, precision, n):
+    """Parameters that start 4 bytes past a 16-byte boundary take the scalar
+    weight loads: the same values, so the same bits."""
+    P = {"f32tc": L.F32_TC, "bf16": L.BF16}[precision]
+    g = torch.Generator(device="cuda").manual_seed(n)
+    k0 = torch.randn(n, 12, generator=g, device="cuda") * 0.3
+    d = torch.nn.functional.normalize(torch.randn(n // 7 + 1, 3, generator=g, device="cuda"), dim=1)
+    ray = (torch.arange(n, device="cuda") // 7).int()
+    up = torch.randn(n, 3, generator=g, device="cuda") * 1e-3
+    p = torch.from_numpy(synth.mlp_params(seed=1)).cuda()
+    shifted = torch.empty(p.numel() + 1, device="cuda")[1:]
+    shifted.copy_(p)
+    assert shifted.data_ptr() % 16 == 4
+    got = []
+    for params in (p, shifted):
+        rgb = torch.empty(n, 3, device="cuda")
+        act = torch.empty(L.rgbnet_act_bytes(n, P), dtype=torch.uint8, device="cuda")
+        g_p, g_k0 = torch.zeros_like(p), torch.empty_like(k0)
+        L.rgbnet_fwd(k0, d, ray, None, n, None, params, P, rgb, act)
+        L.rgbnet_bwd(up, None, None, k0, d, ray, None, n, None, params, P, g_p, g_k0, act, rgb)
+        got.append((rgb, g_p, g_k0))
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n", [1, 129, 152 * 128, 152 * 128 + 1, 305 * 128 + 77])
+def test_proposal_bwd_tile_counts(L, n):
+    """One tile, one per CTA, an odd number per CTA (the two groups of
+    epilogue warps get unequal shares), against torch in 64 bits on the stored
+    BF16 parameters.  A sample whose ReLU input lies within the operands' reach
+    of 0 may switch the unit: its share of the gradient is allowed as slack."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    xyz = torch.rand(n, 3, generator=g, device="cuda") * 2 - 1
+    up = torch.randn(n, generator=g, device="cuda")
+    p = torch.from_numpy(synth.proposal_params(2)).cuda()
+    g_p = torch.zeros_like(p)
+    L.proposal_bwd(up, xyz, None, n, None, p, g_p)
+    assert L.device_status() == 0
+    q = p.to(torch.bfloat16).double().requires_grad_()
+    W1, b1, W2, b2, W3 = q[:2496].view(64, 39), q[2496:2560], q[2560:6656].view(64, 64), q[6656:6720], q[6720:6784]
+    x = xyz.double()
+    arg = (x[:, :, None] * 2.0 ** torch.arange(6, device="cuda", dtype=torch.float64)).flatten(1)
+    z1 = torch.cat([x, arg.sin(), arg.cos()], 1) @ W1.T + b1
+    z2 = torch.relu(z1) @ W2.T + b2
+    z = torch.relu(z2) @ W3 + q[6784]
+    (ref,) = torch.autograd.grad(z, q, up.double(), retain_graph=True)
+    close = torch.minimum(z1.abs().amin(1), z2.abs().amin(1)) < 2e-5
+    slack = torch.zeros_like(ref)
+    for s in close.nonzero()[:, 0].tolist():
+        (gs,) = torch.autograd.grad(z[s], q, up[s].double(), retain_graph=True)
+        slack += 2 * gs.abs()
+    tol = 2e-5 * ref.abs().max()   # two BF16 terms: 2^-16 of each factor
+    assert bool(((g_p.double() - ref).abs() <= tol + slack).all())

@@ -121,3 +121,73 @@ def test_proposal_bwd_tile_counts(L, n):
         slack += 2 * gs.abs()
     tol = 2e-5 * ref.abs().max()   # two BF16 terms: 2^-16 of each factor
     assert bool(((g_p.double() - ref).abs() <= tol + slack).all())
+
+
+@pytest.mark.parametrize("n_flat", [3, 4099, 22019])
+@pytest.mark.parametrize("density", [0.0, 0.03, 0.5, 1.0])
+def test_adam_list_against_single_arrays(L, n_flat, density):
+    """The list kernel (flagged bricks of two grids and a flat vector with a
+    cut last group and a short last block) against the call per array: the same
+    arithmetic, so the same bits; unlisted bricks untouched, flags cleared."""
+    nb, dev = 300, "cuda"
+    g = torch.Generator(device=dev).manual_seed(n_flat)
+    flags = (torch.rand(nb, generator=g, device=dev) < 0.4).to(torch.uint8)
+    lst = torch.empty(nb, dtype=torch.int32, device=dev)
+    cnt = torch.zeros(1, dtype=torch.int32, device=dev)
+    L.touched_compact(flags, nb, lst, cnt)
+
+    def state(n, dens):
+        r = [torch.randn(n, generator=g, device=dev) for _ in range(4)]
+        r[3] = r[3].abs()
+        r[1] = r[1] * (torch.rand(n, generator=g, device=dev) < dens)
+        return r   # p, g, m, v
+    sets = [state(nb * 512, density), state(nb * 512 * 12, density), state(n_flat, 1.0)]
+    sh = torch.zeros(nb * 512 * 12, dtype=torch.bfloat16, device=dev)
+    ref = [[x.clone() for x in s] for s in sets]
+    ref_sh, f = sh.clone(), [flags.clone() for _ in range(4)]
+    step = torch.zeros(2, dtype=torch.int64, device=dev)
+    step[0] = 4
+    L.adam_step_multi_dev(
+        [(s[0], sh if i == 1 else None, *s[1:], s[0].numel(), f[i] if i < 2 else None, 512 * (1, 12, 0)[i], 0.1,
+          *((lst, cnt) if i < 2 else ())) for i, s in enumerate(sets)], 0.9, 0.99, 1e-15, step, True)
+    for i, s in enumerate(ref):
+        L.adam_step(s[0], ref_sh if i == 1 else None, *s[1:], s[0].numel(), f[2 + i] if i < 2 else None,
+                    512 * (1, 12, 0)[i], 0.1, 0.9, 0.99, 1e-15, 5, True)
+    assert int(step[0]) == 5
+    for a, b in zip(sets, ref):
+        for x, y in zip(a, b):
+            assert torch.equal(x, y)
+    assert torch.equal(sh, ref_sh)
+    assert int(f[0].sum()) == 0 and int(f[1].sum()) == 0
+
+
+@pytest.mark.parametrize("G", [(61, 47, 53), (8, 8, 8), (9, 16, 17)])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_tv_pair_against_single_grids(L, G, bf16):
+    """The paired sparse TV over the brick list against the call per grid: the
+    same arithmetic, so the same bits (sides no multiple of the brick, empty
+    and full bricks, entries zero in some channels)."""
+    dev, nb = "cuda", L.grid_num_bricks(G)
+    g = torch.Generator(device=dev).manual_seed(sum(G))
+    flags = (torch.rand(nb, generator=g, device=dev) < 0.7).to(torch.uint8)
+    flags[0] = 1
+    lst = torch.empty(nb, dtype=torch.int32, device=dev)
+    cnt = torch.zeros(1, dtype=torch.int32, device=dev)
+    L.touched_compact(flags, nb, lst, cnt)
+    dt = L.BF16 if bf16 else L.F32
+    grids, ref = [], []
+    for C, w in ((12, 1e-3), (1, 1e-2)):
+        dense = torch.randn(G[2], G[1], G[0], C, generator=g, device=dev).to(torch.bfloat16 if bf16 else torch.float32)
+        p = torch.empty(L.grid_bricked_elems(G, C), dtype=dense.dtype, device=dev)
+        L.grid_pack(dense, p, G, C, dt)
+        up = torch.randn(G[2], G[1], G[0], C, generator=g, device=dev)
+        up = up * (torch.rand(G[2], G[1], G[0], 1, generator=g, device=dev) < 0.3)
+        up = up * (torch.rand(up.shape, generator=g, device=dev) < 0.8)
+        gg = torch.empty(L.grid_bricked_elems(G, C), device=dev)
+        L.grid_pack(up, gg, G, C, L.F32)
+        grids.append((p, dt, C, w, flags, gg))
+        ref.append(gg.clone())
+        L.tv_add_grad(p, dt, G, C, w, 0.5, False, flags, ref[-1])
+    L.tv_add_grad_multi(grids, G, 0.5, False, lst, cnt)
+    for (_, _, _, _, _, gg), r in zip(grids, ref):
+        assert torch.equal(gg, r)

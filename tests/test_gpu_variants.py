@@ -191,3 +191,47 @@ def test_tv_pair_against_single_grids(L, G, bf16):
     L.tv_add_grad_multi(grids, G, 0.5, False, lst, cnt)
     for (_, _, _, _, _, gg), r in zip(grids, ref):
         assert torch.equal(gg, r)
+
+
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 152 * 128 + 5])
+@pytest.mark.parametrize("saved", [True, False])
+def test_rgbnet_f32_tiles(L, n, saved):
+    """The CUDA-core form at tile edges, with and without the stored
+    activations, against torch in 64 bits.  FP32 sums of at most 128 terms: 1e-5
+    of the largest value (a unit whose input lies within 1e-6 of 0 may switch;
+    its samples are set aside, their share of the gradient allowed as slack)."""
+    dev = "cuda"
+    g = torch.Generator(device=dev).manual_seed(n)
+    k0 = torch.randn(n, 12, generator=g, device=dev) * 0.3
+    d = torch.nn.functional.normalize(torch.randn(n // 5 + 1, 3, generator=g, device=dev), dim=1)
+    ray = (torch.arange(n, device=dev) // 5).int()
+    up = torch.randn(n, 3, generator=g, device=dev)
+    p = torch.from_numpy(synth.mlp_params(seed=4)).to(dev)
+    rgb, act = torch.empty(n, 3, device=dev), torch.full((n, 256), -7.0, device=dev) if saved else None
+    g_p, g_k0 = torch.zeros_like(p), torch.empty_like(k0)
+    L.rgbnet_fwd(k0, d, ray, None, n, None, p, L.F32, rgb, act)
+    L.rgbnet_bwd(up, None, None, k0, d, ray, None, n, None, p, L.F32, g_p, g_k0, act, rgb if saved else None)
+    q = p.double().requires_grad_()
+    x0 = k0.double().requires_grad_()
+    at, W = 0, []
+    for s in ((128, 39), (128,), (128, 128), (128,), (3, 128), (3,)):
+        m = int(np.prod(s))
+        W.append(q[at:at + m].view(s))
+        at += m
+    dd = d.double()[ray.long()]
+    arg = (dd[:, :, None] * 2.0 ** torch.arange(4, device=dev, dtype=torch.float64)).flatten(1)
+    z1 = torch.cat([x0, dd, arg.sin(), arg.cos()], 1) @ W[0].T + W[1]
+    z2 = torch.relu(z1) @ W[2].T + W[3]
+    y = torch.sigmoid(torch.relu(z2) @ W[4].T + W[5])
+    r_p, r_k0 = torch.autograd.grad(y, (q, x0), up.double(), retain_graph=True)
+    close = torch.minimum(z1.abs().amin(1), z2.abs().amin(1)) < 1e-6
+    slack = torch.zeros_like(r_p)
+    for s in close.nonzero()[:, 0].tolist():
+        (gs,) = torch.autograd.grad(y[s], q, up[s].double(), retain_graph=True)
+        slack += 2 * gs.abs()
+    assert float((rgb.double() - y).abs().max()) <= 1e-5
+    assert bool(((g_k0.double() - r_k0).abs().amax(1)[~close] <= 1e-5 * r_k0.abs().max()).all())
+    assert bool(((g_p.double() - r_p).abs() <= 1e-5 * r_p.abs().max() + slack).all())
+    if saved:
+        assert float((act[:, :128].double() - torch.relu(z1)).abs().max()) <= 1e-5 * float(z1.abs().max())
+        assert float((act[:, 128:].double() - torch.relu(z2)).abs().max()) <= 1e-5 * float(z2.abs().max())

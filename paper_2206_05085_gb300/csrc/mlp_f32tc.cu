@@ -188,6 +188,7 @@ struct Side {
   uint64_t bar_dw2;   // dW2 done (all H1 terms are free)
   uint64_t bar_gx;    // g_X and dW1 done (G's shared memory and X are free)
   uint64_t bar_fin;   // every product done (before the accumulators are read)
+  uint64_t rows_full; // the next tile's g_z3 and scales in shared memory (4 warp arrivals)
   uint64_t g2a_full;  // G2 of the first half of the rows in tensor memory (16 warp arrivals)
   uint64_t g2_full;   // G2 of a tile in tensor and shared memory (16 warp arrivals)
   uint64_t g1_full;   // G1 of a tile in tensor and shared memory (16 warp arrivals)
@@ -1007,6 +1008,7 @@ __global__ void __launch_bounds__(kThreads, 1) rgbnet_bwd_tc_kernel(
     tc::mbar_init(&fs->bar_dw2, 1);
     tc::mbar_init(&fs->bar_gx, 1);
     tc::mbar_init(&fs->bar_fin, 1);
+    tc::mbar_init(&fs->rows_full, 4);
     tc::mbar_init(&fs->g2a_full, 16);
     tc::mbar_init(&fs->g2_full, 16);
     tc::mbar_init(&fs->g1_full, 16);
@@ -1316,7 +1318,7 @@ __global__ void __launch_bounds__(kThreads, 1) rgbnet_bwd_tc_kernel(
     for (int64_t k = 0; k < nt; ++k) {
       if (qw < 2) up_l1(up, idx, tile_of(k + 1) * kTile + row, n);
       m1b = m1b_next;
-      tc::named_sync(1, 512);   // every row's g_z3 and scales are in shared memory
+      if (k > 0) bwd_wait(fs, &fs->rows_full, (uint32_t)(k - 1) & 1u);   // g_z3 and scales of the tile's rows
       bwd_wait(fs, &fs->bar_d2, ph_d2);
       ph_d2 ^= 1;
       tc::fence_after_sync();
@@ -1399,7 +1401,11 @@ __global__ void __launch_bounds__(kThreads, 1) rgbnet_bwd_tc_kernel(
       tc::fence_after_sync();
       // every warp has passed its G2 epilogue (bar_gh follows g2_full): the
       // rows of this tile have been read
-      if (qw == 1 && k + 1 < nt) row_store(k + 1);
+      if (qw == 1 && k + 1 < nt) {
+        row_store(k + 1);
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&fs->rows_full);
+      }
       // G1 = g_h1 * (H1 > 0): at S1 in shared memory (dW1), at sG1 in tensor
       // memory (g_X), in two halves of 16 hidden units
       const uint32_t e = fs->sc[k & 1][row];

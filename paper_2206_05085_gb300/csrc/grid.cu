@@ -224,65 +224,42 @@ __device__ __forceinline__ void mark_touched(uint8_t* touched, const TriArgs& T,
   if (sx && sy && sz) touched[brick_of(T.g, x1, y1, z1)] = 1;
 }
 
-template <int C>
-__global__ void __launch_bounds__(256) scatter_bwd_kernel(const float* __restrict__ g_out, TriArgs T,
-                                                          const float* __restrict__ xyz,
-                                                          const int32_t* __restrict__ idx,
-                                                          int64_t n_cap, const int64_t* n_dev,
-                                                          float* __restrict__ g_grid,
-                                                          uint8_t* __restrict__ touched) {
-  const int64_t n = live_n(n_cap, n_dev);
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n;
-       j += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t s = idx ? (int64_t)__ldg(idx + j) : j;
-    Corners c;
-    corners(T, xyz, s, c);
-    float go[C];
-    if constexpr (C % 4 == 0) {
-#pragma unroll
-      for (int q = 0; q < C / 4; ++q) {
-        float4 v = __ldg(reinterpret_cast<const float4*>(g_out + s * C) + q);
-        go[4 * q] = v.x;
-        go[4 * q + 1] = v.y;
-        go[4 * q + 2] = v.z;
-        go[4 * q + 3] = v.w;
-      }
-    } else {
-#pragma unroll
-      for (int ch = 0; ch < C; ++ch) go[ch] = __ldg(g_out + s * C + ch);
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      float* p = g_grid + c.slot[k] * C;
-      if constexpr (C % 4 == 0) {
-#pragma unroll
-        for (int q = 0; q < C / 4; ++q)
-          atomicAdd(reinterpret_cast<float4*>(p) + q,
-                    make_float4(c.w[k] * go[4 * q], c.w[k] * go[4 * q + 1], c.w[k] * go[4 * q + 2],
-                                c.w[k] * go[4 * q + 3]));
-      } else {
-#pragma unroll
-        for (int ch = 0; ch < C; ++ch) atomicAdd(p + ch, c.w[k] * go[ch]);
-      }
-    }
-    mark_touched(touched, T, c);
-  }
-}
+// Density (1 channel, kA) and feature (12 channels, kB) adjoints, in one pass
+// when both are given, warp-aggregated: a warp takes 32 consecutive list
+// positions, and two neighbouring lanes whose samples lie in the same grid
+// cell (consecutive samples of a ray often do) are merged into one set of
+// reductions for both.  Pairs are formed greedily along each run of equal
+// cells.  The features then go out one merged sample per instruction: its
+// eight corners times three float4 on 24 lanes, so that a voxel's 48 bytes
+// (and its x neighbour's, where both lie in one pair of the Morton order)
+// reach the L2 as whole sectors.  What bounds it: the L2's rate of sector
+// reductions.  A lane per sample, one float4 of a voxel per instruction (the
+// form before), touched each sector up to three times: pair 75 -> 53 us on
+// 160^3, 381 -> 267 us on 320^3 contracted, 107 -> 72 us on a 384 x 384 x 256
+// stack, 53 -> 33 us on 64^3; 12 channels alone, 762,026 samples on 160^3 and
+// unmerged before, 96 -> 48 us, one channel 24 -> 15 us.
+struct ScatterStage {
+  float4 gb[32][3];
+  int64_t slot[32][8];
+  float w[32][8];
+  float ga[32];
+  uint8_t rep[32];
+};
 
-// Density (1 channel) and feature (12 channels) adjoints in one pass,
-// warp-aggregated: a warp takes 32 consecutive list positions, and two
-// neighbouring lanes whose samples lie in the same grid cell (consecutive
-// samples of a ray often do) are merged - the first lane adds the second
-// lane's weighted gradients to its own and issues one set of reductions for
-// both.  Pairs are formed greedily along each run of equal cells.
-__global__ void __launch_bounds__(256) scatter_bwd_1_12_kernel(
+template <bool kA, bool kB>
+__global__ void __launch_bounds__(256) scatter_merge_kernel(
     const float* __restrict__ g_a, float* __restrict__ grid_a, uint8_t* __restrict__ touched_a,
     const float* __restrict__ g_b, float* __restrict__ grid_b, uint8_t* __restrict__ touched_b, TriArgs T,
     const float* __restrict__ xyz, const int32_t* __restrict__ idx, int64_t n_cap, const int64_t* n_dev) {
+  __shared__ ScatterStage stages[kB ? 8 : 1];
+  ScatterStage& st = stages[kB ? threadIdx.x >> 5 : 0];
   const int64_t n = live_n(n_cap, n_dev);
   const int lane = threadIdx.x & 31;
   const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  // over half a sample per voxel: the density's reductions are spread between
+  // the features' (bursts of them meet in the few sectors they have)
+  const bool crowded = 2 * n > (int64_t)T.g.G[0] * T.g.G[1] * T.g.G[2];
   for (int64_t j0 = warp0 * 32; j0 < n; j0 += nwarps * 32) {
     const int64_t j = j0 + lane;
     const bool valid = j < n;
@@ -294,14 +271,16 @@ __global__ void __launch_bounds__(256) scatter_bwd_1_12_kernel(
     if (valid) {
       const int64_t s = idx ? (int64_t)__ldg(idx + j) : j;
       corners(T, xyz, s, c);
-      ga = __ldg(g_a + s);
+      if (kA) ga = __ldg(g_a + s);
+      if (kB) {
 #pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const float4 v = __ldg(reinterpret_cast<const float4*>(g_b + s * 12) + q);
-        gb[4 * q] = v.x;
-        gb[4 * q + 1] = v.y;
-        gb[4 * q + 2] = v.z;
-        gb[4 * q + 3] = v.w;
+        for (int q = 0; q < 3; ++q) {
+          const float4 v = __ldg(reinterpret_cast<const float4*>(g_b + s * 12) + q);
+          gb[4 * q] = v.x;
+          gb[4 * q + 1] = v.y;
+          gb[4 * q + 2] = v.z;
+          gb[4 * q + 3] = v.w;
+        }
       }
       key = c.slot[0];
     } else {
@@ -312,34 +291,85 @@ __global__ void __launch_bounds__(256) scatter_bwd_1_12_kernel(
       }
     }
     // lanes continuing the previous lane's cell; greedy pairing along runs
+    // (a lane is absorbed when an odd number of such steps ends at it)
     const int64_t prev = __shfl_up_sync(0xffffffffu, key, 1);
     const unsigned same = __ballot_sync(0xffffffffu, lane > 0 && prev == key);
-    unsigned absorbed = 0u;
-    for (int i = 1; i < 32; ++i)
-      if (((same >> i) & 1u) && !((absorbed >> (i - 1)) & 1u)) absorbed |= 1u << i;
-    // the next lane's weights and gradients (used when it is absorbed into this one)
-    float wn[8], gan, gbn[12];
+    // lane's distance from its run's start: the lanes below it, down to the first that starts a run
+    const unsigned starts = ~same & (lane == 31 ? 0xffffffffu : (2u << lane) - 1u);
+    const bool absorbed = ((lane - (31 - __clz(starts))) & 1) != 0;
+    const unsigned abs_mask = __ballot_sync(0xffffffffu, absorbed);
+    if constexpr (!kB) {
+      // one channel: the lane issues its cell's eight reductions
+      float wn[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) wn[k] = __shfl_down_sync(0xffffffffu, c.w[k], 1);
-    gan = __shfl_down_sync(0xffffffffu, ga, 1);
+      for (int k = 0; k < 8; ++k) wn[k] = __shfl_down_sync(0xffffffffu, c.w[k], 1);
+      const float gan = __shfl_down_sync(0xffffffffu, ga, 1);
+      if (!valid || absorbed) continue;
+      const bool pair = lane < 31 && ((abs_mask >> (lane + 1)) & 1u);
 #pragma unroll
-    for (int i = 0; i < 12; ++i) gbn[i] = __shfl_down_sync(0xffffffffu, gb[i], 1);
-    if (!valid || ((absorbed >> lane) & 1u)) continue;
-    const bool pair = lane < 31 && ((absorbed >> (lane + 1)) & 1u);
+      for (int k = 0; k < 8; ++k) atomicAdd(grid_a + c.slot[k], fmaf(pair ? wn[k] : 0.0f, gan, c.w[k] * ga));
+      mark_touched(touched_a, T, c);
+    } else {
+      __syncwarp();   // the last step's rows have been read
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const float w0 = c.w[k], w1 = pair ? wn[k] : 0.0f;
-      atomicAdd(grid_a + c.slot[k], fmaf(w1, gan, w0 * ga));
-      float4* p = reinterpret_cast<float4*>(grid_b + c.slot[k] * 12);
+      for (int k = 0; k < 8; ++k) {
+        st.w[lane][k] = c.w[k];
+        st.slot[lane][k] = c.slot[k];
+      }
 #pragma unroll
       for (int q = 0; q < 3; ++q)
-        atomicAdd(p + q, make_float4(fmaf(w1, gbn[4 * q], w0 * gb[4 * q]),
-                                     fmaf(w1, gbn[4 * q + 1], w0 * gb[4 * q + 1]),
-                                     fmaf(w1, gbn[4 * q + 2], w0 * gb[4 * q + 2]),
-                                     fmaf(w1, gbn[4 * q + 3], w0 * gb[4 * q + 3])));
+        st.gb[lane][q] = make_float4(gb[4 * q], gb[4 * q + 1], gb[4 * q + 2], gb[4 * q + 3]);
+      if (kA) st.ga[lane] = ga;
+      const unsigned reps = __ballot_sync(0xffffffffu, valid && !absorbed);
+      if (valid && !absorbed) {
+        // the merged sample's row, and in bit 7 whether the next lane's is added
+        const bool pair = lane < 31 && ((abs_mask >> (lane + 1)) & 1u);
+        st.rep[__popc(reps & ((1u << lane) - 1u))] = (uint8_t)(lane | (pair ? 128 : 0));
+        if (kA) mark_touched(touched_a, T, c);
+        mark_touched(touched_b, T, c);
+      }
+      __syncwarp();
+      const int nr = __popc(reps);
+      auto density = [&](int e, int k) {   // corner k of the merged sample e
+        const int r = e & 31;
+        float v = st.w[r][k] * st.ga[r];
+        if (e & 128) v = fmaf(st.w[r + 1][k], st.ga[r + 1], v);
+        atomicAdd(grid_a + st.slot[r][k], v);
+      };
+      // corner k's channels 4 q .. + 3 of the merged sample e
+      auto feature = [&](int e, int k, int q) {
+        const int r = e & 31;
+        const float w0 = st.w[r][k];
+        const float4 g0 = st.gb[r][q];
+        float4 v = make_float4(w0 * g0.x, w0 * g0.y, w0 * g0.z, w0 * g0.w);
+        if (e & 128) {
+          const float w1 = st.w[r + 1][k];
+          const float4 g1 = st.gb[r + 1][q];
+          v = make_float4(fmaf(w1, g1.x, v.x), fmaf(w1, g1.y, v.y), fmaf(w1, g1.z, v.z), fmaf(w1, g1.w, v.w));
+        }
+        atomicAdd(reinterpret_cast<float4*>(grid_b + st.slot[r][k] * 12) + q, v);
+      };
+      // one merged sample after the other: lane 3 k + q takes its corner k, channels 4 q ..
+      const int k3 = lane / 3, q3 = lane - 3 * k3;
+      if (kA && crowded) {   // lanes 24-31 the density's corners beside it
+        for (int i = 0; i < nr; ++i) {
+          if (lane < 24)
+            feature(st.rep[i], k3, q3);
+          else
+            density(st.rep[i], lane - 24);
+        }
+      } else {
+        if (lane < 24)
+          for (int i = 0; i < nr; ++i) feature(st.rep[i], k3, q3);
+        // the density on its own: four merged samples at a time, the four a
+        // quarter of the list apart (neighbours would meet in one voxel)
+        if (kA) {
+          const int per = (nr + 3) >> 2, at = (lane >> 3) * per;
+          for (int i = 0; i < per; ++i)
+            if (at + i < nr) density(st.rep[at + i], lane & 7);
+        }
+      }
     }
-    mark_touched(touched_a, T, c);
-    mark_touched(touched_b, T, c);
   }
 }
 
@@ -1324,8 +1354,12 @@ extern "C" int dvgo_sample_grid_bwd(const float* g_out, const dvgo_grid_desc* gd
   cudaStream_t st = as_stream(stream);
   const int block = 256;
   int g = grid_for(n_cap, block, 16);
-  if (C == 1) scatter_bwd_kernel<1><<<g, block, 0, st>>>(g_out, T, xyz, idx, n_cap, n_dev, g_grid, touched);
-  else if (C == 12) scatter_bwd_kernel<12><<<g, block, 0, st>>>(g_out, T, xyz, idx, n_cap, n_dev, g_grid, touched);
+  if (C == 1)
+    scatter_merge_kernel<true, false><<<g, block, 0, st>>>(g_out, g_grid, touched, nullptr, nullptr, nullptr, T, xyz,
+                                                           idx, n_cap, n_dev);
+  else if (C == 12)
+    scatter_merge_kernel<false, true><<<g, block, 0, st>>>(nullptr, nullptr, nullptr, g_out, g_grid, touched, T, xyz,
+                                                           idx, n_cap, n_dev);
   else scatter_bwd_generic_kernel<<<g, block, 0, st>>>(g_out, T, C, xyz, idx, n_cap, n_dev, g_grid, touched);
   return launch_status();
 }
@@ -1424,7 +1458,7 @@ extern "C" int dvgo_sample_grid_bwd2(const float* g_out_a, int32_t C_a, float* g
     TriArgs T;
     DVGO_CHECK_ARG(make_tri(T, gd));
     cudaStream_t st = as_stream(stream);
-    scatter_bwd_1_12_kernel<<<grid_for(n_cap, 256, 16), 256, 0, st>>>(
+    scatter_merge_kernel<true, true><<<grid_for(n_cap, 256, 16), 256, 0, st>>>(
         g_out_a, g_grid_a, touched_a, g_out_b, g_grid_b, touched_b, T, xyz, idx, n_cap, n_dev);
     return launch_status();
   }

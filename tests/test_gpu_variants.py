@@ -235,3 +235,54 @@ def test_rgbnet_f32_tiles(L, n, saved):
     if saved:
         assert float((act[:, :128].double() - torch.relu(z1)).abs().max()) <= 1e-5 * float(z1.abs().max())
         assert float((act[:, 128:].double() - torch.relu(z2)).abs().max()) <= 1e-5 * float(z2.abs().max())
+
+
+@pytest.mark.parametrize("G", [(9, 10, 11), (64, 40, 33)])   # crowded (over half a sample per voxel) and not
+@pytest.mark.parametrize("n", [1, 31, 33, 257, 4099])
+@pytest.mark.parametrize("form", ["a", "b", "ab"])
+def test_scatter_merge(L, G, n, form):
+    """The merged adjoints (one channel, twelve, both) on runs of samples in one
+    cell, an index list with a device count below the capacity, against a 64-bit
+    scatter.  FP32 sums of at most n terms per voxel: 1e-5 of the largest entry."""
+    dev = "cuda"
+    g = torch.Generator(device=dev).manual_seed(n + G[0])
+    base = torch.rand(n // 3 + 1, 3, generator=g, device=dev) * 2.2 - 1.1      # some outside the box
+    xyz = (base.repeat_interleave(3, 0)[:n] + 0.01 * torch.rand(n, 3, generator=g, device=dev)).contiguous()
+    ga = torch.randn(n, generator=g, device=dev)
+    gb = torch.randn(n, 12, generator=g, device=dev)
+    idx = torch.arange(n, device=dev, dtype=torch.int32).flip(0).contiguous()
+    m = n - n // 5
+    n_dev = torch.tensor([m], dtype=torch.int64, device=dev)
+    gd = L.GridDesc.make(-1.0, 1.0, G)
+    out = [torch.zeros(L.grid_bricked_elems(G, C), device=dev) for C in (1, 12)]
+    flags = [torch.zeros(L.grid_num_bricks(G), dtype=torch.uint8, device=dev) for _ in range(2)]
+    if form == "ab":
+        L.sample_grid_bwd2(ga, 1, out[0], flags[0], gb, 12, out[1], flags[1], gd, xyz, idx, n, n_dev)
+    elif form == "a":
+        L.sample_grid_bwd(ga, gd, 1, xyz, idx, n, n_dev, out[0], flags[0])
+    else:
+        L.sample_grid_bwd(gb, gd, 12, xyz, idx, n, n_dev, out[1], flags[1])
+    sel = idx[:m].long()
+    dim = torch.tensor(G, device=dev)
+    u = ((xyz[sel].double() + 1) * 0.5 * (dim - 1)).clamp(min=0)
+    u = torch.minimum(u, (dim - 1).double())
+    i = torch.minimum(u.floor().long(), dim - 2)
+    f = u - i
+    for C, up, got, fl in ((1, ga[:, None], out[0], flags[0]), (12, gb, out[1], flags[1])):
+        ref = torch.zeros(G[2] * G[1] * G[0], C, dtype=torch.float64, device=dev)
+        if {1: "a", 12: "b"}[C] in form:
+            for k in range(8):
+                o = torch.tensor([k & 1, (k >> 1) & 1, k >> 2], device=dev)
+                w = torch.where(o.bool(), f, 1 - f).prod(1, keepdim=True)
+                c = i + o
+                ref.index_add_(0, (c[:, 2] * G[1] + c[:, 1]) * G[0] + c[:, 0], w * up[sel].double())
+        dense = torch.empty(G[2], G[1], G[0], C, device=dev)
+        L.grid_unpack(got, dense, G, C, L.F32)
+        assert float((dense.view(-1, C).double() - ref).abs().max()) <= 1e-5 * max(float(ref.abs().max()), 1.0)
+        hit = torch.zeros(G[2], G[1], G[0], dtype=torch.bool, device=dev)
+        hit[(ref.abs().amax(1) > 0).view(G[2], G[1], G[0])] = True
+        nb = [(x + 7) // 8 for x in G]
+        full = torch.zeros(8 * nb[2], 8 * nb[1], 8 * nb[0], dtype=torch.bool, device=dev)
+        full[:G[2], :G[1], :G[0]] = hit
+        want = full.view(nb[2], 8, nb[1], 8, nb[0], 8).permute(0, 2, 4, 1, 3, 5).reshape(-1, 512).any(1)
+        assert bool((fl.bool() | ~want).all())    # every brick with a contribution is flagged

@@ -320,19 +320,8 @@ __device__ __forceinline__ void mma3_ts16(uint32_t d, uint32_t a_tmem, uint32_t 
   }
 }
 
-// 16 values times s split into the 16-column chunk layout of mma3_ts16: hi
-// terms of value pairs in words 0-7, lo terms in words 8-15.
-template <class Op>
-__device__ __forceinline__ void split16(const float (&v)[16], float s, uint32_t (&hl)[16], float& vmax) {
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const float a = s * v[2 * c], b = s * v[2 * c + 1];
-    vmax = fmaxf(vmax, fmaxf(fabsf(a), fabsf(b)));
-    hl[c] = Op::split2(a, b, hl[8 + c]);
-  }
-}
-
-// The split terms of split16 times r (a power of two <= 1) as the hi / lo
+// 16 values' split terms (the 16-column chunks of mma3_ts16: hi terms of value
+// pairs in words 0-7, lo terms in 8-15) times r (a power of two <= 1) as the hi / lo
 // core-matrix rows of columns k0 .. k0 + 15 of row `row` in shared memory.
 template <class Op, bool kScale = true>
 __device__ __forceinline__ void st_terms16(uint8_t* hi, uint8_t* lo, int row, int k0, const uint32_t (&hl)[16],
@@ -573,6 +562,8 @@ __device__ __forceinline__ float enc_col(int q, int c, float d0, float d1, float
 // distinct ray of the warp's 32 rows (consecutive samples mostly share a ray):
 // for up to 8 distinct rays, lane 8 j' + c evaluates column c of the j-th
 // ray (4 rays per round) and each row collects its 8 columns by shuffles.
+// (The leaders' lanes come from votes: __fns is a loop, and cost 5 % of the
+// whole forward: 317 and 301 us for 1.9e6 samples.)
 __device__ __forceinline__ void quarter_x_shared(const RowIn& in, int q, int lane, float v[16]) {
   const int key = in.s >= 0 ? in.r : -1;
   const unsigned peers = __match_any_sync(0xffffffffu, key);
@@ -586,9 +577,16 @@ __device__ __forceinline__ void quarter_x_shared(const RowIn& in, int q, int lan
 #pragma unroll
   for (int k = 0; k < 16; ++k) v[k] = 0.0f;
   const int rank = __popc(leaders & ((1u << leader) - 1u));
+  // lane of the j-th distinct ray's leader (-1 past the last one)
+  auto nth = [&](int j) { return __ffs(__ballot_sync(0xffffffffu, lane == leader && rank == j)) - 1; };
   for (int r0 = 0; r0 < nd; r0 += 4) {
-    const int j = min(r0 + (lane >> 3), nd - 1), c = lane & 7;
-    const int src = (int)__fns(leaders, 0, j + 1);
+    const int c = lane & 7;
+    int src = nth(r0);
+    if (nd > r0 + 1) {
+      const int g = lane >> 3, s1 = nth(r0 + 1), s2 = nth(r0 + 2), s3 = nth(r0 + 3);
+      const int t = g == 1 ? s1 : (g == 2 ? s2 : (g == 3 ? s3 : src));
+      src = t >= 0 ? t : src;   // (past the last ray: any)
+    }
     const float d0 = __shfl_sync(0xffffffffu, in.d[0], src);
     const float d1 = __shfl_sync(0xffffffffu, in.d[1], src);
     const float d2 = __shfl_sync(0xffffffffu, in.d[2], src);
@@ -627,9 +625,14 @@ static_assert(gEnd + sizeof(FwdSide) + 2 * 4 * kTile * kOut * sizeof(float) <= 2
               "forward shared memory");
 
 // Bounded wait shared by all roles of the forward; after the first timeout
-// every later wait returns false immediately, so that all threads still
-// reach the same barriers and the kernel ends.
+// every later wait on a phase that is not complete returns false immediately,
+// so that all threads still reach the same barriers and the kernel ends.
+// The barrier is polled before the abort word is read: while the tensor core
+// and the bulk copies read shared memory one such read takes some 300 cycles
+// (both orders measured at 1.9e6 samples: forward 301 and 296 us, backward
+// 578 and 552 us).
 __device__ __forceinline__ bool fwd_wait(FwdSide* fs, uint64_t* bar, uint32_t parity) {
+  if (tc::mbar_try_wait(bar, parity)) return true;
   if (*reinterpret_cast<volatile int*>(&fs->abort)) return false;
   if (tc::mbar_wait(bar, parity, kSpin)) return true;
   *reinterpret_cast<volatile int*>(&fs->abort) = 1;
@@ -651,6 +654,17 @@ __device__ __forceinline__ bool fwd_wait(FwdSide* fs, uint64_t* bar, uint32_t pa
 // The tile image in the act buffer (the layout the backward loads) is written
 // by bulk copies that the MMA warp issues: X from its buffer, H1 from a
 // shared-memory staging copy that the compute warps fill beside the TMEM one.
+// What bounds it: latency along a tile's chain (MMA issue after the last
+// warp's arrival, the H1 epilogue, the next layer 1) with the issue slots
+// half used; every shared-memory read of a wait or an epilogue queues behind
+// the operands and the image copies.  From about 10 tiles a CTA on the image
+// also goes to HBM, 90 KB a tile (at 1.9e6 samples 1.3 GB in 296 us; without
+// those writes 282 us before, of 317).  Measured, FP32 form: 393,909 samples
+// 77.7 us before the waits and the leader search were shortened and 75 us
+// now, 1.9e6 samples 317 and 296 us, BF16 form 786,433 samples 141 and 131 us.
+// Issuing layer 1 of tile k + 1 before layer 2 of tile k, deferring the output
+// layer's cross-quarter sum and fetching features by asynchronous copies were
+// each measured and gave nothing more.
 // Before the layer-1 MMAs of tile k are committed the MMA thread waits until
 // those copies have read their sources, so l1_full(k) also tells the compute
 // warps that the staging area and X buffer k & 1 may be rewritten.
@@ -914,8 +928,8 @@ __global__ void __launch_bounds__(kThreads, 1) rgbnet_fwd_tc_kernel(
 // column quarter's warps for all) and form its relu mask.  Epilogue arithmetic
 // is packed (two FP32 values per instruction), G2 is split once and its
 // second copy formed by multiplying the 16-bit terms.  Measured, 1.9e6
-// samples, FP32 form: 782 us before, 582 us now (393,909 samples: 197 and
-// 152 us; 1003 samples with the partial sums: 31.8 and 25.7 us).
+// samples, FP32 form: 782 us before, 552 us now (393,909 samples: 197 and
+// 150 us; 1003 samples with the partial sums: 31.8 and 25.5 us).
 //
 // Order per tile t of this CTA (tn = the next one):
 //   compute: wait d2(t) -> G2 of the rows 32 q .. + 15; wait gx(t - 1) ->
@@ -971,9 +985,10 @@ __device__ __forceinline__ void up_l3(UpIn& u, const float* __restrict__ g_rgb,
   for (int c = 0; c < kOut; ++c) u.g[c] = u.g[c] * y[c] * (1.0f - y[c]);
 }
 
-// Bounded wait of the backward; after the first timeout every later wait
-// returns false at once, so that both roles still reach the kernel's end.
+// Bounded wait of the backward, as fwd_wait: after the first timeout both
+// roles still reach the kernel's end.
 __device__ __forceinline__ bool bwd_wait(Side* fs, uint64_t* bar, uint32_t parity) {
+  if (tc::mbar_try_wait(bar, parity)) return true;
   if (*reinterpret_cast<volatile int*>(&fs->abort)) return false;
   if (tc::mbar_wait(bar, parity, kSpin)) return true;
   *reinterpret_cast<volatile int*>(&fs->abort) = 1;

@@ -178,6 +178,8 @@ struct Side {
   // Rows 2p, 2p + 1 of the tile: g_z3[0] of both, then [1], [2], each times
   // the row's own gradient scale sG2, then the two 1 / sG2.
   float4 smp[kTile / 2][2];
+  // S2 / sG2 of every row as a term (a power of two)
+  alignas(16) uint16_t fac[kTile];
   uint16_t sc[2][kTile];   // by tile parity: exponent fields of a row's sG2 (low byte) and sG1
   uint32_t tiny[4];   // rows 32 q ..: some row's S2 / sG2 is below the factor a term can be multiplied by
   uint64_t bar_h;     // H1 terms of a tile image landed
@@ -920,7 +922,7 @@ __global__ void __launch_bounds__(kThreads, 1) rgbnet_fwd_tc_kernel(
 //
 // What bounds it: the epilogues and the waits between them (one tile's
 // operands fill the shared memory, so a tile's phases follow one another; the
-// MMAs are 5.6k cycles of a tile's ~12k).  So the order puts as much as it
+// MMAs are 5.6k cycles of a tile's ~10k).  So the order puts as much as it
 // can beside the G2 epilogue and the wait for g_h1: dW2 runs in two halves
 // (the rows of an epilogue half each), the first beside the second epilogue
 // half; the next tile's H1 terms are copied in per half, as dW2 frees them;
@@ -928,8 +930,8 @@ __global__ void __launch_bounds__(kThreads, 1) rgbnet_fwd_tc_kernel(
 // column quarter's warps for all) and form its relu mask.  Epilogue arithmetic
 // is packed (two FP32 values per instruction), G2 is split once and its
 // second copy formed by multiplying the 16-bit terms.  Measured, 1.9e6
-// samples, FP32 form: 782 us before, 552 us now (393,909 samples: 197 and
-// 150 us; 1003 samples with the partial sums: 31.8 and 25.5 us).
+// samples, FP32 form: 782 us before, 530 us now (393,909 samples: 197 and
+// 142 us; 1003 samples with the partial sums: 31.8 and 25.1 us).
 //
 // Order per tile t of this CTA (tn = the next one):
 //   compute: wait d2(t) -> G2 of the rows 32 q .. + 15; wait gx(t - 1) ->
@@ -1114,6 +1116,7 @@ __global__ void __launch_bounds__(kThreads, 1) rgbnet_bwd_tc_kernel(
     q[2] = rowg[1];
     q[4] = rowg[2];
     q[6] = rowr;
+    fs->fac[row] = (uint16_t)Op::pack(S2 * rowr, 0.0f);
     fs->sc[k & 1][row] = (uint16_t)rowe;
     const bool any = __any_sync(0xffffffffu, rowtiny);
     if (lane == 0) fs->tiny[warp & 3] = any ? 1u : 0u;
@@ -1345,7 +1348,12 @@ __global__ void __launch_bounds__(kThreads, 1) rgbnet_bwd_tc_kernel(
       // of g_h1), and with its terms times S2 / sG2 (the CTA-wide scale S2)
       // into tensor memory over the half's own D2 columns (lane = unit, K =
       // row: the A operand of dW2).  A factor too small for the term format
-      // (a row 2^-24 below the CTA's largest) takes a split of its own.
+      // (a row 2^-24 below the CTA's largest) takes a split of its own, in a
+      // rolled loop over the terms in shared memory: this epilogue is on every
+      // tile's critical cycle (G2 -> dW2, g_h1 and the next D2^T -> G2), and
+      // the unrolled rare path in its middle and the factors formed per thread
+      // cost 4 % (1.9e6 samples 552 and 530 us, BF16 form 786,433 samples 276
+      // and 248 us).
       const bool tiny = fs->tiny[qw] != 0u;
 #pragma unroll 1
       for (int h = 0; h < 2; ++h) {
@@ -1376,20 +1384,30 @@ __global__ void __launch_bounds__(kThreads, 1) rgbnet_bwd_tc_kernel(
           tc::fence_after_sync();
         }
         st_terms16<Op, false>(sm + bGh, sm + bGl, oh, r0, hl, 1.0f);
+        if (!tiny) {   // (warp-uniform)
+          const uint4 fa = *reinterpret_cast<const uint4*>(fs->fac + r0),
+                      fb = *reinterpret_cast<const uint4*>(fs->fac + r0 + 8);
+          const uint32_t fac[8] = {fa.x, fa.y, fa.z, fa.w, fb.x, fb.y, fb.z, fb.w};
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const float2 q = reinterpret_cast<const float2*>(&fs->smp[(r0 >> 1) + c][1])[1];
-          const f32x2 f2 = mul2(S2x, pack2(q.x, q.y));
-          if (tiny) {
-            hl[c] = split_pair<Op>(mul2(Op::join2(hl[c], hl[8 + c]), f2), hl[8 + c], vmax);
-          } else {
-            const float2 f = unpack2(f2);
-            const uint32_t fac = Op::pack(f.x, f.y);
-            hl[c] = Op::mul2v(hl[c], fac);
-            hl[8 + c] = Op::mul2v(hl[8 + c], fac);
+          for (int c = 0; c < 8; ++c) {
+            hl[c] = Op::mul2v(hl[c], fac[c]);
+            hl[8 + c] = Op::mul2v(hl[8 + c], fac[c]);
+          }
+          tc::tmem_st16(lane_base + cTmp + r0, hl);
+        } else {   // rare: from the terms in shared memory, one pair a step (little code)
+#pragma unroll 1
+          for (int c = 0; c < 8; ++c) {
+            const uint32_t off = tc::cm_off(oh, r0 + 2 * c, kSboH);
+            const float2 q = reinterpret_cast<const float2*>(&fs->smp[(r0 >> 1) + c][1])[1];
+            const f32x2 f2 = mul2(S2x, pack2(q.x, q.y));
+            const f32x2 g = Op::join2(*reinterpret_cast<const uint32_t*>(sm + bGh + off),
+                                      *reinterpret_cast<const uint32_t*>(sm + bGl + off));
+            uint32_t lo;
+            const uint32_t hi = split_pair<Op>(mul2(g, f2), lo, vmax);
+            tc::tmem_st1(lane_base + cTmp + r0 + c, hi);
+            tc::tmem_st1(lane_base + cTmp + r0 + 8 + c, lo);
           }
         }
-        tc::tmem_st16(lane_base + cTmp + r0, hl);
         if (h == 1 && k > 0 && qw == 0) store_gx();
         tc::tmem_wait_st();
         tc::fence_proxy_async_smem();

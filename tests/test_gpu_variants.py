@@ -286,3 +286,25 @@ def test_scatter_merge(L, G, n, form):
         full[:G[2], :G[1], :G[0]] = hit
         want = full.view(nb[2], 8, nb[1], 8, nb[0], 8).permute(0, 2, 4, 1, 3, 5).reshape(-1, 512).any(1)
         assert bool((fl.bool() | ~want).all())    # every brick with a contribution is flagged
+
+
+@pytest.mark.parametrize("shift", [0, 1], ids=["aligned", "unaligned"])
+@pytest.mark.parametrize("R", [1, 31, 1023, 1024, 1025, 8192, 8193, 152 * 1024 + 1, 400_001])
+def test_count_scan_blocks(L, R, shift):
+    """Live-sample list over per-ray counts whose scan is split over blocks:
+    one to three passes a block, a last block of one ray, counts off 16-byte
+    alignment."""
+    rng = np.random.default_rng(R)
+    cand = rng.integers(0, 6, R)
+    live = np.minimum(rng.integers(0, 6, R), cand).astype(np.int32)
+    off = np.concatenate([[0], np.cumsum(cand)]).astype(np.int64)
+    seg = torch.from_numpy(np.concatenate([np.zeros(shift, np.int32), live])).cuda()[shift:]
+    n = int(live.sum())
+    idx = torch.full((max(n, 1),), -1, dtype=torch.int32, device="cuda")
+    count = torch.zeros(1, dtype=torch.int64, device="cuda")
+    ws = torch.empty(L.live_samples_workspace_size(R), dtype=torch.uint8, device="cuda")
+    L.live_samples(torch.from_numpy(off).cuda(), seg, R, idx, count, ws)
+    assert int(count) == n
+    dst = np.concatenate([[0], np.cumsum(live)])[:-1]
+    want = np.arange(n) + np.repeat(off[:-1] - dst, live)
+    assert np.array_equal(idx.cpu().numpy()[:n], want)

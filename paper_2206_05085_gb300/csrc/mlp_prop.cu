@@ -364,10 +364,9 @@ __global__ void __launch_bounds__(128, kFwdPerSM) prop_fwd_kernel(const float* _
 //   stage 1: D = H1 W2^T
 //   stage 2: dW2 += G2^T H1;  db2 += G2^T 1 (X's ones column);  D = G2 W2
 //   stage 3: dW1|db1 += G1^T X
-// The MMA warp takes whichever group's stage is ready, so that one group's
-// epilogues go beside the other's MMAs (a fixed order two stages apart made
-// each group wait 40 % of its time); the weight gradients of both sum in one
-// set of accumulators.  g_params += the CTA's sums (atomics at the end).
+// The groups run two stages apart, so that one's epilogues go beside the
+// other's MMAs; the weight gradients of both sum in one set of accumulators,
+// tile after tile.  g_params += the CTA's sums (atomics at the end).
 // What bounds it: the epilogues (about 650 instructions a thread and tile);
 // the MMAs are 2.8k cycles a tile.  The weight gradients are M = 64 products
 // (32 cycles each for N = 64; the 128-row form with the gradient padded to
@@ -409,32 +408,20 @@ __global__ void __launch_bounds__(kBwdThreads, 1) prop_bwd_kernel(const float* _
   if (warp == 16) {
     // ------------------------------------------------------- MMA issuer
     const uint32_t sW1 = tc::smem_u32(sm + bW1), sW2 = tc::smem_u32(sm + bW2);
-    // stages of each group in order, the group whose operands are in first (of
-    // two, the one on a short stage); dW2, db2 and dW1 start with the first
-    // stage that adds to them
-    int64_t left[2] = {4 * ((tiles + 1) / 2), 4 * (tiles / 2)};
-    uint32_t at[2] = {0u, 0u};   // stages done
-    bool dw2 = false, dw1 = false;
-    while (left[0] + left[1] > 0) {
-      int g = -1;
+    uint32_t ph[2] = {0u, 0u};
+    bool ok = true;
+    // stage `st` of tile k (group k & 1) once its operands are in (lane 0 polls)
+    auto stage = [&](int64_t k, int st) {
+      if (!ok || k < 0 || k >= tiles) return;
+      const int g = (int)(k & 1);
+      int r = 0;
       if (lane == 0) {
-        for (uint32_t it = 0; it < kSpin && g < 0 && !*(volatile int*)&fs->error; ++it) {
-          const bool r0 = left[0] > 0 && tc::mbar_test(&fs->ready[0], at[0] & 1u);
-          const bool r1 = left[1] > 0 && tc::mbar_test(&fs->ready[1], at[1] & 1u);
-          if (r0 || r1) g = r0 && (!r1 || (at[0] & 3u) < 2u) ? 0 : 1;
-        }
-        if (g < 0) atomicExch(&fs->error, 1);
+        r = !*(volatile int*)&fs->error && tc::mbar_wait(&fs->ready[g], ph[g], kSpin) ? 1 : 0;
+        if (!r) atomicExch(&fs->error, 1);
       }
-      g = __shfl_sync(0xffffffffu, g, 0);
-      if (g < 0) break;
-      const int st = (int)((g ? at[1] : at[0]) & 3u);
-      if (g) {
-        ++at[1];
-        --left[1];
-      } else {
-        ++at[0];
-        --left[0];
-      }
+      ph[g] ^= 1;
+      ok = __shfl_sync(0xffffffffu, r, 0) != 0;
+      if (!ok) return;
       tc::fence_after_sync();
       if (tc::elect_one()) {
         const uint32_t base = tc::smem_u32(sm + bGroup) + (uint32_t)g * kGroupBytes, D = tmem + cD + kH * (uint32_t)g;
@@ -456,14 +443,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) prop_bwd_kernel(const float* _
             dw += (2 * kSboW2) >> 4;
           }
           mma_grad(tmem + cDW2, base + oGh, base + oGl, base + oHh, base + oHl, kSboH, tc::idesc_bf16(64, kH, 1, 1),
-                   dw2);
+                   k > 0);
           // db2: X's columns 32-47 hold the exact ones column
           uint64_t gh = tc::smem_desc_mn(base + oGh, kSboH, 128), gl = tc::smem_desc_mn(base + oGl, kSboH, 128);
           uint64_t dx = tc::smem_desc_mn(base + oXh + 4 * 128, kSboX, 128);
           const uint32_t id16 = tc::idesc_bf16(64, 16, 1, 1);
 #pragma unroll
           for (int q = 0; q < kTile / 16; ++q) {
-            tc::mma_bf16(tmem + cDB2, gh, dx, id16, (dw2 || q > 0) ? 1u : 0u);
+            tc::mma_bf16(tmem + cDB2, gh, dx, id16, (k > 0 || q > 0) ? 1u : 0u);
             tc::mma_bf16(tmem + cDB2, gl, dx, id16, 1u);
             gh += (2 * kSboH) >> 4;
             gl += (2 * kSboH) >> 4;
@@ -471,13 +458,24 @@ __global__ void __launch_bounds__(kBwdThreads, 1) prop_bwd_kernel(const float* _
           }
         } else {
           mma_grad(tmem + cDW1, base + oGh, base + oGl, base + oXh, base + oXl, kSboX, tc::idesc_bf16(64, kK1, 1, 1),
-                   dw1);
+                   k > 0);
         }
         tc::mma_commit(&fs->gdone[g]);
       }
       __syncwarp();
-      dw2 = dw2 || st == 2;
-      dw1 = dw1 || st == 3;
+    };
+    // group 0 on tile k (even), group 1 two stages behind it on tile k + 1
+    stage(0, 0);
+    stage(0, 1);
+    for (int64_t k = 0; k < tiles; k += 2) {
+      stage(k, 2);
+      stage(k + 1, 0);
+      stage(k, 3);
+      stage(k + 1, 1);
+      stage(k + 2, 0);
+      stage(k + 1, 2);
+      stage(k + 2, 1);
+      stage(k + 1, 3);
     }
     // every MMA issued has finished before tensor memory is read or released
     if (tc::elect_one()) {

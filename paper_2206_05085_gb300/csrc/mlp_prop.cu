@@ -247,7 +247,8 @@ using namespace prop;
 // phases of a tile follow one another; four resident CTAs per SM (H1 stays in
 // tensor memory, so a CTA needs 39 KB of shared memory and 128 TMEM columns)
 // fill each other's waits.  What bounds it: the encoding and the epilogues on
-// the CUDA cores (about 1.5k instructions a row).
+// the CUDA cores (about 1.5k instructions a row).  Measured, 5.3e6
+// candidates: 615 us with H1 in shared memory and two CTAs per SM, 324 us now.
 __global__ void __launch_bounds__(128, kFwdPerSM) prop_fwd_kernel(const float* __restrict__ xyz,
                                                                   const int32_t* __restrict__ idx, int64_t n_cap,
                                                                   const int64_t* __restrict__ n_dev,
@@ -371,7 +372,12 @@ __global__ void __launch_bounds__(128, kFwdPerSM) prop_fwd_kernel(const float* _
 // the MMAs are 2.8k cycles a tile.  The weight gradients are M = 64 products
 // (32 cycles each for N = 64; the 128-row form with the gradient padded to
 // 128 took 48); dW3 is summed per thread over all tiles and reduced over the
-// rows once.
+// rows once.  Measured, 5.3e6 candidates: 2605 us with one group, 128-row
+// gradients and rolled issue loops; 840 us in this form with waits that read
+// the error word before the barrier (a shared-memory round trip on every
+// stage's chain), 813 us with the barrier polled first.  An MMA warp that polls
+// both groups and takes whichever is ready is slower (914 us): its polling
+// competes for shared memory.
 __global__ void __launch_bounds__(kBwdThreads, 1) prop_bwd_kernel(const float* __restrict__ g_out,
                                                                   const float* __restrict__ xyz,
                                                                   const int32_t* __restrict__ idx, int64_t n_cap,
@@ -416,7 +422,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) prop_bwd_kernel(const float* _
       const int g = (int)(k & 1);
       int r = 0;
       if (lane == 0) {
-        r = !*(volatile int*)&fs->error && tc::mbar_wait(&fs->ready[g], ph[g], kSpin) ? 1 : 0;
+        r = tc::mbar_try_wait(&fs->ready[g], ph[g]) ||
+                    (!*(volatile int*)&fs->error && tc::mbar_wait(&fs->ready[g], ph[g], kSpin))
+                ? 1
+                : 0;
         if (!r) atomicExch(&fs->error, 1);
       }
       ph[g] ^= 1;
@@ -495,7 +504,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) prop_bwd_kernel(const float* _
       if (lane == 0) tc::mbar_arrive(&fs->ready[group]);
     };
     auto await = [&]() -> bool {   // the outcome is the warp's
-      const bool ok = !*(volatile int*)&fs->error && tc::mbar_wait(&fs->gdone[group], ph, kSpin);
+      const bool ok = tc::mbar_try_wait(&fs->gdone[group], ph) ||
+                      (!*(volatile int*)&fs->error && tc::mbar_wait(&fs->gdone[group], ph, kSpin));
       ph ^= 1;
       if (!ok) atomicExch(&fs->error, 1);
       const bool all = __all_sync(0xffffffffu, ok);

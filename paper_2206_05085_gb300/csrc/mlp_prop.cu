@@ -57,7 +57,7 @@ constexpr uint32_t oXh = 0, oXl = oXh + kXBytes, oHh = oXl + kXBytes, oHl = oHh 
 constexpr uint32_t cD = 0, cDW2 = 128, cDW1 = 192, cDB2 = 240;
 
 struct Side {
-  float2 ob[kH];    // per hidden unit: (b2, W3)
+  alignas(16) float2 ob[kH];    // per hidden unit: (b2, W3)
   float b3;
   uint64_t ready[2];   // backward, per group: its operands of the next stage are written (8 warps)
   uint64_t gdone[2];   // backward, per group: MMAs of the stage finished
@@ -248,7 +248,9 @@ using namespace prop;
 // tensor memory, so a CTA needs 39 KB of shared memory and 128 TMEM columns)
 // fill each other's waits.  What bounds it: the encoding and the epilogues on
 // the CUDA cores (about 1.5k instructions a row).  Measured, 5.3e6
-// candidates: 615 us with H1 in shared memory and two CTAs per SM, 324 us now.
+// candidates: 615 us with H1 in shared memory and two CTAs per SM, 324 us now;
+// a tile's rows on twice the warps (half the encoding and the columns each)
+// took 328 us, so it is the instructions and not their latency.
 __global__ void __launch_bounds__(128, kFwdPerSM) prop_fwd_kernel(const float* __restrict__ xyz,
                                                                   const int32_t* __restrict__ idx, int64_t n_cap,
                                                                   const int64_t* __restrict__ n_dev,
@@ -341,9 +343,10 @@ __global__ void __launch_bounds__(128, kFwdPerSM) prop_fwd_kernel(const float* _
       float v[32];
       tc::tmem_ld32(lane_base + kH + ch * 32, v);
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        const float2 q = fs->ob[ch * 32 + i];
+      for (int i = 0; i < 32; i += 2) {
+        const float4 q = *reinterpret_cast<const float4*>(&fs->ob[ch * 32 + i]);
         z = fmaf(q.y, fmaxf(v[i] + q.x, 0.0f), z);
+        z = fmaf(q.w, fmaxf(v[i + 1] + q.z, 0.0f), z);
       }
     }
     if (j < n) out[idx ? (int64_t)__ldg(idx + j) : j] = z;
@@ -375,7 +378,8 @@ __global__ void __launch_bounds__(128, kFwdPerSM) prop_fwd_kernel(const float* _
 // rows once.  Measured, 5.3e6 candidates: 2605 us with one group, 128-row
 // gradients and rolled issue loops; 840 us in this form with waits that read
 // the error word before the barrier (a shared-memory round trip on every
-// stage's chain), 813 us with the barrier polled first.  An MMA warp that polls
+// stage's chain), 813 us with the barrier polled first, 804 us with the output
+// layer's constants read for two units at a time.  An MMA warp that polls
 // both groups and takes whichever is ready is slower (914 us): its polling
 // competes for shared memory.
 __global__ void __launch_bounds__(kBwdThreads, 1) prop_bwd_kernel(const float* __restrict__ g_out,
@@ -556,11 +560,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1) prop_bwd_kernel(const float* _
         float v[16];
         tc::tmem_ld16(Dt + 16 * c, v);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const float2 q = fs->ob[32 * half + 16 * c + i];
-          const float z2 = v[i] + q.x;
-          dW3acc[16 * c + i] = fmaf(gup, fmaxf(z2, 0.0f), dW3acc[16 * c + i]);
-          v[i] = z2 > 0.0f ? gup * q.y : 0.0f;
+        for (int i = 0; i < 16; i += 2) {
+          const float4 q = *reinterpret_cast<const float4*>(&fs->ob[32 * half + 16 * c + i]);
+          const float z0 = v[i] + q.x, z1 = v[i + 1] + q.z;
+          dW3acc[16 * c + i] = fmaf(gup, fmaxf(z0, 0.0f), dW3acc[16 * c + i]);
+          dW3acc[16 * c + i + 1] = fmaf(gup, fmaxf(z1, 0.0f), dW3acc[16 * c + i + 1]);
+          v[i] = z0 > 0.0f ? gup * q.y : 0.0f;
+          v[i + 1] = z1 > 0.0f ? gup * q.w : 0.0f;
         }
 #pragma unroll
         for (int q = 0; q < 2; ++q) st_split8(gb + oGh, gb + oGl, row, 32 * half + 16 * c + 8 * q, kSboH, v + 8 * q);

@@ -1582,9 +1582,14 @@ __global__ void __launch_bounds__(256) partials_reduce_kernel(const float* __res
   const int per = (rows + 7) / 8, b0 = grp * per, b1 = std::min(rows, b0 + per);
   float a = 0.0f;
   if (p < kNumParams) {
-#pragma unroll 8
-    for (int b = b0; b < b1; ++b) a += __ldg(p < kPartRow ? part + (size_t)b * kPartRow + p
-                                                          : part + (size_t)kNumSMs * kPartRow + b * kOut + p - kPartRow);
+    const float* src = p < kPartRow ? part + p : part + (size_t)kNumSMs * kPartRow + p - kPartRow;
+    const int stride = p < kPartRow ? kPartRow : kOut;
+    constexpr int kPer = (kNumSMs + 7) / 8;
+    float v[kPer];   // all of the group's rows in flight at once
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) v[i] = b0 + i < b1 ? __ldg(src + (size_t)(b0 + i) * stride) : 0.0f;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) a += v[i];
   }
   acc[grp][j] = a;
   __syncthreads();

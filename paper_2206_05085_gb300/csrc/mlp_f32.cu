@@ -20,7 +20,9 @@
 // 130,000 samples: forward 170 us with scalar FMAs in 8 x 8 blocks on 8 warps
 // (half the FMA pipe idle on dependences), 141 us packed in 4 x 8 blocks of
 // 32 x 16 threads (12 wavefronts per 16 packed FMAs: bandwidth), 137 us in this
-// form; backward 362, 317 and 308 us.
+// form with the X tile built by four warps between two barriers, 127 us with
+// each warp building its own rows (250,000 samples: 248 and 225 us); backward
+// 362, 317 and 300 us.
 #include "common.cuh"
 #include "mlp_common.cuh"
 
@@ -170,6 +172,51 @@ __device__ __forceinline__ void build_x_tile(float* XS, const float* __restrict_
   }
 }
 
+// What a lane of the forward loads for its tile row (row lane / 4 of the warp's
+// eight, q = lane % 4): features 4 q .. + 3 (q < 3) and the ray's direction.
+// The loads depend on each other (list index; feature row and ray id;
+// direction), so they are issued in three steps, spread over the tile before.
+struct XRow {
+  int64_t s;   // sample index (-1 past the list end)
+  int32_t r;
+  float4 f;
+  float d[3];
+  __device__ __forceinline__ void l1(const int32_t* __restrict__ idx, int64_t j, int64_t n) {
+    s = j < n ? (idx ? (int64_t)__ldg(idx + j) : j) : -1;
+  }
+  __device__ __forceinline__ void l2(const float* __restrict__ k0, const int32_t* __restrict__ ray_id, int q) {
+    f = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    r = -1;
+    if (s < 0) return;
+    if (q < 3) f = __ldg(reinterpret_cast<const float4*>(k0 + s * kFeat) + q);
+    r = __ldg(ray_id + s);
+  }
+  __device__ __forceinline__ void l3(const float* __restrict__ rays_d) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) d[a] = r >= 0 ? __ldg(rays_d + 3 * (int64_t)r + a) : 0.0f;
+  }
+  // This lane's part of the input row (the row of encode_row): its features
+  // (q = 3: the direction and the constant) and the pairs p = 3 q .. + 2.
+  __device__ __forceinline__ void store(float* x, int q) const {
+    const bool valid = s >= 0;
+    if (q < 3) {
+      st4(x + 4 * q, f);
+    } else {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) x[kFeat + a] = d[a];
+      x[kIn] = valid ? 1.0f : 0.0f;
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const int p = 3 * q + i, a = p >> 2;
+      float sn, cs;
+      sincosf((a == 0 ? d[0] : (a == 1 ? d[1] : d[2])) * (float)(1 << (p & 3)), &sn, &cs);
+      x[kFeat + 3 + p] = valid ? sn : 0.0f;
+      x[kFeat + 3 + 3 * kNumFreq + p] = valid ? cs : 0.0f;
+    }
+  }
+};
+
 __global__ void __launch_bounds__(kF32Threads, 1) rgbnet_fwd_f32_kernel(
     const float* __restrict__ k0, const float* __restrict__ rays_d,
     const int32_t* __restrict__ ray_id, const int32_t* __restrict__ idx, int64_t n_cap,
@@ -195,13 +242,20 @@ __global__ void __launch_bounds__(kF32Threads, 1) rgbnet_fwd_f32_kernel(
     for (int c = 0; c < 3; ++c) w3[c][b] = __ldg(params + kOffW3 + c * kHid + 4 * lane + b);
   }
   const float4 b2v = make_float4(b2a[0], b2a[1], b2a[2], b2a[3]), zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int xq = lane & 3, xrow = kRowsT * warp + (lane >> 2);
+  XRow xr;
+  xr.l1(idx, (int64_t)blockIdx.x * kTile + xrow, n);
+  xr.l2(k0, ray_id, xq);
+  xr.l3(rays_d);
+  __syncthreads();   // the weights are in; from here on a warp touches its own eight rows only
   for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
     const int64_t j0 = t * kTile;
-    __syncthreads();
-    build_x_tile(XS, k0, rays_d, ray_id, idx, j0, n);
-    __syncthreads();
+    xr.store(XS + xrow * kP40, xq);
+    xr.l1(idx, j0 + (int64_t)gridDim.x * kTile + xrow, n);   // the next tile's rows
+    __syncwarp();
     f32x2 acc[kRowsT][2];
     gemm_nn<kInP>(XS, kP40, W1T, kP128, acc);
+    xr.l2(k0, ray_id, xq);
 #pragma unroll
     for (int a = 0; a < kRowsT; ++a) {
       const int r = kRowsT * warp + a;
@@ -211,6 +265,7 @@ __global__ void __launch_bounds__(kF32Threads, 1) rgbnet_fwd_f32_kernel(
     }
     __syncwarp();   // a warp reads back only its own rows
     gemm_nn<kHid>(HS, kP128, W2T, kP128, acc);
+    xr.l3(rays_d);
     // layer 3: 8 rows x 3 outputs of the warp, reduced over its lanes (lane l
     // ends with row l / 3, output l % 3)
     float z[32];

@@ -447,36 +447,35 @@ __global__ void __launch_bounds__(kF32Threads, 1) rgbnet_bwd_f32_kernel(
       }
     }
     __syncthreads();  // g_z2 no longer read
-    // g_k0[s][k] = sum_o g_z1[s][o] W1[o][k], k < 12: rows ty + 32a, k = tx
-    auto store_gk0 = [&]() {
-      if (tx >= kFeat) return;
+    // The x tile is built by the first 128 threads while the 384 others form
+    // g_k0[s][k] = sum_o g_z1[s][o] W1[o][k], k < 12: rows g + 32a of one column.
+    if (tid < kTile) {
+      build_x_tile(GS, k0, rays_d, ray_id, idx, j0, n);
+    } else {
+      static_assert(kF32Threads - kTile == 32 * kFeat, "32 row groups of one thread per column");
+      const int g = (tid - kTile) / kFeat, k = (tid - kTile) % kFeat;
       float gk[4];
 #pragma unroll
       for (int a = 0; a < 4; ++a) gk[a] = 0.0f;
 #pragma unroll 2
       for (int o = 0; o < kHid; o += 4) {
-        const float w0 = W1S[o * kP40 + tx], w1 = W1S[(o + 1) * kP40 + tx];
-        const float w2 = W1S[(o + 2) * kP40 + tx], w3v = W1S[(o + 3) * kP40 + tx];
+        const float w0 = W1S[o * kP40 + k], w1 = W1S[(o + 1) * kP40 + k];
+        const float w2 = W1S[(o + 2) * kP40 + k], w3v = W1S[(o + 3) * kP40 + k];
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
-          const float4 g = ld4(H1S + (ty + 32 * a) * kP128 + o);
-          gk[a] = fmaf(g.x, w0, fmaf(g.y, w1, fmaf(g.z, w2, fmaf(g.w, w3v, gk[a]))));
+          const float4 q = ld4(H1S + (g + 32 * a) * kP128 + o);
+          gk[a] = fmaf(q.x, w0, fmaf(q.y, w1, fmaf(q.z, w2, fmaf(q.w, w3v, gk[a]))));
         }
       }
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
-        const int64_t j = j0 + ty + 32 * a;
+        const int64_t j = j0 + g + 32 * a;
         if (j < n) {
           const int64_t s = idx ? (int64_t)__ldg(idx + j) : j;
-          g_k0[s * kFeat + tx] = gk[a];
+          g_k0[s * kFeat + k] = gk[a];
         }
       }
-    };
-    // the x tile is built by the first 128 threads while the others form their g_k0
-    if (tid < kTile)
-      build_x_tile(GS, k0, rays_d, ray_id, idx, j0, n);
-    else
-      store_gk0();
+    }
     __syncthreads();
     // dW1[o][k] += sum_s g_z1[s][o] x[s][k]; o in {2ty.., 64+2ty..}, k in {tx, tx+16, tx+32}
     {
@@ -506,7 +505,6 @@ __global__ void __launch_bounds__(kF32Threads, 1) rgbnet_bwd_f32_kernel(
         x2 = y2;
       }
     }
-    if (tid < kTile) store_gk0();
   }
   // flush partials
 #pragma unroll

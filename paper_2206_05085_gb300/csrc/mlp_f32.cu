@@ -22,7 +22,8 @@
 // 32 x 16 threads (12 wavefronts per 16 packed FMAs: bandwidth), 137 us in this
 // form with the X tile built by four warps between two barriers, 127 us with
 // each warp building its own rows (250,000 samples: 248 and 225 us); backward
-// 362, 317 and 300 us.
+// 362, 317 and 300 us (292 with g_k0 on the threads that do not build the
+// input tile; dW1 in 2 x 5 blocks, with fewer wavefronts, was not faster).
 #include "common.cuh"
 #include "mlp_common.cuh"
 

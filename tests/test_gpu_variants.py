@@ -308,3 +308,35 @@ def test_count_scan_blocks(L, R, shift):
     dst = np.concatenate([[0], np.cumsum(live)])[:-1]
     want = np.arange(n) + np.repeat(off[:-1] - dst, live)
     assert np.array_equal(idx.cpu().numpy()[:n], want)
+
+
+@pytest.mark.parametrize("steps", [1, 7, 8, 61, 130, 512])
+@pytest.mark.parametrize("R", [1, 31, 33, 300])
+def test_contracted_fill_groups(L, R, steps):
+    """The contracted march's second pass from checkpoints (eight steps at a
+    time, a warp writing four rays at once) against the march that writes as
+    it goes: chunks shorter than a group, remainders, a ragged last block,
+    sparse and full occupancy."""
+    cfg = synth.CONFIGS["unbounded_320"]
+    rp = synth.render_params(cfg)
+    sd = L.SamplerDesc()
+    sd.mode, sd.near, sd.max_steps = 1, rp.near, steps
+    sd.contract_b, sd.p_inf, sd.step_c = rp.contract_b, steps % 2, rp.step_c * 4
+    gd = L.GridDesc.make(cfg.bbox_min, cfg.bbox_max, [40] * 3)
+    o, d = (torch.from_numpy(np.ascontiguousarray(v)).cuda() for v in synth.rays(cfg, seed=R, n_rays=R))
+    n = R * steps
+    for mask in (None, (torch.rand(40, 40, 40, generator=torch.Generator().manual_seed(1)) < 0.4)
+                 .to(torch.uint8).cuda()):
+        outs = []
+        for _ in range(2):
+            outs.append([torch.full((R + 1,), -1, dtype=torch.int64, device="cuda"),
+                         torch.full((n, 3), -1.0, device="cuda"),
+                         torch.full((n,), -1, dtype=torch.int32, device="cuda"),
+                         torch.full((n,), -1, dtype=torch.int32, device="cuda"),
+                         torch.full((n,), -1.0, device="cuda"), torch.full((n,), -1.0, device="cuda")])
+        ws = torch.empty(L.sample_rays_workspace_size(R), dtype=torch.uint8, device="cuda")
+        L.sample_rays(o, d, R, gd, sd, mask, n, *outs[0], ws)
+        L.sample_rays_noalloc(o, d, R, gd, sd, mask, n, *outs[1])
+        assert int(outs[0][0][-1]) > 0 or mask is not None
+        for a, b in zip(*outs):
+            assert torch.equal(a, b)

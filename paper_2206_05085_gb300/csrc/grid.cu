@@ -307,7 +307,11 @@ __global__ void __launch_bounds__(256) scatter_merge_kernel(
       if (!valid || absorbed) continue;
       const bool pair = lane < 31 && ((abs_mask >> (lane + 1)) & 1u);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) atomicAdd(grid_a + c.slot[k], fmaf(pair ? wn[k] : 0.0f, gan, c.w[k] * ga));
+      for (int k = 0; k < 8; ++k) {   // (a neighbour that is not merged is left out, not weighted by 0: it may be infinite)
+        float v = c.w[k] * ga;
+        if (pair) v = fmaf(wn[k], gan, v);
+        atomicAdd(grid_a + c.slot[k], v);
+      }
       mark_touched(touched_a, T, c);
     } else {
       __syncwarp();   // the last step's rows have been read

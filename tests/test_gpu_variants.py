@@ -288,6 +288,52 @@ def test_scatter_merge(L, G, n, form):
         assert bool((fl.bool() | ~want).all())    # every brick with a contribution is flagged
 
 
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+@pytest.mark.parametrize("form", ["a", "b", "ab"])
+def test_scatter_merge_nonfinite_rows(L, form, bad):
+    """A row whose gradient is infinite or NaN reaches the eight voxels of its
+    own cell and no others, wherever it stands in a warp's 32 samples and in a
+    run of samples of one cell: the other voxels are the finite rows' 64-bit
+    scatter (as in test_scatter_merge: 1e-5 of the largest entry)."""
+    dev, G, n = "cuda", (40, 33, 35), 1003
+    g = torch.Generator(device=dev).manual_seed(5)
+    base = torch.rand(n, 3, generator=g, device=dev) * 1.9 - 0.95
+    run = torch.randint(0, n, (n,), generator=g, device=dev).sort().values     # runs of one to several samples a cell
+    xyz = (base[run] + 0.001 * torch.rand(n, 3, generator=g, device=dev)).contiguous()
+    ga, gb = torch.randn(n, generator=g, device=dev), torch.randn(n, 12, generator=g, device=dev)
+    rows = torch.arange(7, n, 37, device=dev)      # every position modulo 32
+    fin_a, fin_b = ga.clone(), gb.clone()
+    fin_a[rows], fin_b[rows] = 0.0, 0.0
+    ga[rows], gb[rows] = bad, bad
+    gd = L.GridDesc.make(-1.0, 1.0, G)
+    out = [torch.zeros(L.grid_bricked_elems(G, C), device=dev) for C in (1, 12)]
+    if form == "ab":
+        L.sample_grid_bwd2(ga, 1, out[0], None, gb, 12, out[1], None, gd, xyz, None, n, None)
+    elif form == "a":
+        L.sample_grid_bwd(ga, gd, 1, xyz, None, n, None, out[0], None)
+    else:
+        L.sample_grid_bwd(gb, gd, 12, xyz, None, n, None, out[1], None)
+    dim = torch.tensor(G, device=dev)
+    u = (xyz.double() + 1) * 0.5 * (dim - 1)
+    i = u.floor().long()
+    f = u - i
+    for C, up, got in ((1, fin_a[:, None], out[0]), (12, fin_b, out[1])):
+        if {1: "a", 12: "b"}[C] not in form:
+            continue
+        ref = torch.zeros(G[2] * G[1] * G[0], C, dtype=torch.float64, device=dev)
+        own = torch.zeros(G[2] * G[1] * G[0], dtype=torch.bool, device=dev)   # voxels of the bad rows' cells
+        for k in range(8):
+            o = torch.tensor([k & 1, (k >> 1) & 1, k >> 2], device=dev)
+            w = torch.where(o.bool(), f, 1 - f).prod(1, keepdim=True)
+            at = ((i + o)[:, 2] * G[1] + (i + o)[:, 1]) * G[0] + (i + o)[:, 0]
+            ref.index_add_(0, at, w * up.double())
+            own[at[rows]] = True
+        dense = torch.empty(G[2], G[1], G[0], C, device=dev)
+        L.grid_unpack(got, dense, G, C, L.F32)
+        diff = (dense.view(-1, C).double() - ref).abs()[~own]
+        assert bool((diff <= 1e-5 * float(ref.abs().max())).all())     # (NaN compares false)
+
+
 @pytest.mark.parametrize("shift", [0, 1], ids=["aligned", "unaligned"])
 @pytest.mark.parametrize("R", [1, 31, 1023, 1024, 1025, 8192, 8193, 152 * 1024 + 1, 400_001])
 def test_count_scan_blocks(L, R, shift):

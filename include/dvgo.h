@@ -33,6 +33,10 @@
  *    order of the 512 voxels inside a brick, channels innermost.
  *    dvgo_grid_pack/unpack convert from/to the dense layout
  *    g[((z*Gy + y)*Gx + x)*C + c].
+ *  - Buffers need their element type's own alignment and no more, except
+ *    where a call states a rule (then checked on the host).  Trilinear
+ *    queries of 12 channels and their adjoints are faster with rows and
+ *    grids that start on 16-byte boundaries (BF16 grids: 8-byte).
  *
  * Which calls are the operations of the method, and which are fusions:
  *  - The operations (one call each, each the plain form of one step):
@@ -407,7 +411,7 @@ int dvgo_rgb_loss(const float* color, const float* target, const float* L_r, int
  * act: DVGO_F32 may be NULL, else see dvgo_rgbnet_bwd; DVGO_F32_TC and
  * DVGO_BF16 required, dvgo_rgbnet_act_bytes(n_cap, precision) bytes,
  * 16-byte aligned (the forward stores each 128-sample tile's split layer
- * inputs for the backward). */
+ * inputs for the backward).  k0 16-byte aligned. */
 int dvgo_rgbnet_fwd(const float* k0, const float* rays_d, const int32_t* ray_id,
                     const int32_t* idx, int64_t n_cap, const int64_t* n_dev, const float* params,
                     int precision, float* rgb, float* act, void* stream);
@@ -416,7 +420,7 @@ int dvgo_rgbnet_fwd(const float* k0, const float* rays_d, const int32_t* ray_id,
  * [.., 3] at the sample index) when g_rgb is given, else w[s] *
  * g_color[ray_id[s]] (the colour part of the compositing gradient).
  * Accumulates g_params (+=, f32) and writes g_k0 [.., 12] rows at the
- * sample index.  act (FP32 form, may be NULL): f32 [n_cap][256] written by
+ * sample index (k0, g_k0 16-byte aligned).  act (FP32 form, may be NULL): f32 [n_cap][256] written by
  * dvgo_rgbnet_fwd for the same list, row j = [h1 (128) | h2 (128)] of list
  * position j; with it (and rgb, the forward's output, may be NULL) the
  * backward reads the hidden activations instead of recomputing them.
@@ -534,7 +538,8 @@ int dvgo_touched_compact(const uint8_t* touched, int64_t nb, int32_t* list, int3
  * left untouched.  With touched (uint8 per block of block_elems entries,
  * may be NULL) only flagged blocks are visited.  zero_grad != 0 clears the
  * visited gradients and the visited flags.  p_shadow (may be NULL) receives
- * a BF16 copy of every updated p. */
+ * a BF16 copy of every updated p.  With touched: p, g, m, v 16-byte aligned,
+ * p_shadow 8-byte aligned, block_elems a multiple of 4. */
 int dvgo_adam_step(float* p, uint16_t* p_shadow, float* g, float* m, float* v, int64_t n,
                    uint8_t* touched, int64_t block_elems, float lr, float beta1, float beta2,
                    float eps, int64_t step, int zero_grad, void* stream);

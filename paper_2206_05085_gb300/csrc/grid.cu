@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(256) gather_fwd_kernel(const void* __restrict_
   }
 }
 
-// Any channel count (scalar loads).
+// Any channel count and alignment (scalar loads).
 template <bool kBF16>
 __global__ void gather_fwd_generic_kernel(const void* __restrict__ grid, TriArgs T, int C,
                                           const float* __restrict__ xyz,
@@ -1320,7 +1320,10 @@ extern "C" int dvgo_sample_grid_fwd(const void* grid, int dtype, const dvgo_grid
   cudaStream_t st = as_stream(stream);
   const int block = 256;
   int g = grid_for(n_cap, block, 16);
-  if (C == 1 || C == 12) {   // the specialised kernels loop: one resident wave of blocks
+  // 12 channels by 16-byte rows (BF16 grids: 8-byte) where the buffers allow it, else one value at a time
+  const bool special =
+      C == 1 || (C == 12 && (uintptr_t)grid % (dtype == DVGO_F32 ? 16 : 8) == 0 && (uintptr_t)out % 16 == 0);
+  if (special) {   // the specialised kernels loop: one resident wave of blocks
     static int per_sm[2][2] = {{0, 0}, {0, 0}};
     const int di = dtype == DVGO_F32 ? 0 : 1, ci = C == 1 ? 0 : 1;
     if (!per_sm[di][ci]) {
@@ -1336,11 +1339,11 @@ extern "C" int dvgo_sample_grid_fwd(const void* grid, int dtype, const dvgo_grid
   }
   if (dtype == DVGO_F32) {
     if (C == 1) gather_fwd_kernel<1, false><<<g, block, 0, st>>>(grid, T, xyz, idx, n_cap, n_dev, out);
-    else if (C == 12) gather_fwd_kernel<12, false><<<g, block, 0, st>>>(grid, T, xyz, idx, n_cap, n_dev, out);
+    else if (special) gather_fwd_kernel<12, false><<<g, block, 0, st>>>(grid, T, xyz, idx, n_cap, n_dev, out);
     else gather_fwd_generic_kernel<false><<<g, block, 0, st>>>(grid, T, C, xyz, idx, n_cap, n_dev, out);
   } else {
     if (C == 1) gather_fwd_kernel<1, true><<<g, block, 0, st>>>(grid, T, xyz, idx, n_cap, n_dev, out);
-    else if (C == 12) gather_fwd_kernel<12, true><<<g, block, 0, st>>>(grid, T, xyz, idx, n_cap, n_dev, out);
+    else if (special) gather_fwd_kernel<12, true><<<g, block, 0, st>>>(grid, T, xyz, idx, n_cap, n_dev, out);
     else gather_fwd_generic_kernel<true><<<g, block, 0, st>>>(grid, T, C, xyz, idx, n_cap, n_dev, out);
   }
   return launch_status();
@@ -1361,7 +1364,7 @@ extern "C" int dvgo_sample_grid_bwd(const float* g_out, const dvgo_grid_desc* gd
   if (C == 1)
     scatter_merge_kernel<true, false><<<g, block, 0, st>>>(g_out, g_grid, touched, nullptr, nullptr, nullptr, T, xyz,
                                                            idx, n_cap, n_dev);
-  else if (C == 12)
+  else if (C == 12 && (uintptr_t)g_out % 16 == 0 && (uintptr_t)g_grid % 16 == 0)   // rows and voxels by float4
     scatter_merge_kernel<false, true><<<g, block, 0, st>>>(nullptr, nullptr, nullptr, g_out, g_grid, touched, T, xyz,
                                                            idx, n_cap, n_dev);
   else scatter_bwd_generic_kernel<<<g, block, 0, st>>>(g_out, T, C, xyz, idx, n_cap, n_dev, g_grid, touched);

@@ -334,6 +334,47 @@ def test_scatter_merge_nonfinite_rows(L, form, bad):
         assert bool((diff <= 1e-5 * float(ref.abs().max())).all())     # (NaN compares false)
 
 
+def _off_by(t, shift):
+    """t's values in a view that starts `shift` elements past a 16-byte boundary."""
+    v = torch.empty(t.numel() + shift, dtype=t.dtype, device=t.device)[shift:]
+    v.copy_(t.reshape(-1))
+    assert v.data_ptr() % 16 == shift * t.element_size()
+    return v
+
+
+@pytest.mark.parametrize("which", ["grid", "rows", "both"])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_query12_off_alignment(L, bf16, which):
+    """The 12-channel query and its adjoints (single and paired) on grids and
+    rows that start one element past a 16-byte boundary: such buffers take the
+    one-value-at-a-time kernels.  FP32 sums of 8 products (query) and of at most
+    n terms (adjoint): 1e-6 and 1e-5 of the largest value."""
+    dev, G, n = "cuda", (21, 18, 25), 2055
+    g = torch.Generator(device=dev).manual_seed(8)
+    xyz = (torch.rand(n, 3, generator=g, device=dev) * 2.2 - 1.1).contiguous()
+    gd = L.GridDesc.make(-1.0, 1.0, G)
+    dt, tdt = (L.BF16, torch.bfloat16) if bf16 else (L.F32, torch.float32)
+    grid = torch.randn(L.grid_bricked_elems(G, 12), generator=g, device=dev).to(tdt)
+    sg, sr = int(which != "rows"), int(which != "grid")
+    want, got = torch.empty(n * 12, device=dev), _off_by(torch.zeros(n * 12, device=dev), sr)
+    L.sample_grid_fwd(grid, dt, gd, 12, xyz, None, n, None, want)
+    L.sample_grid_fwd(_off_by(grid, sg), dt, gd, 12, xyz, None, n, None, got)
+    assert float((got - want).abs().max()) <= 1e-6 * float(want.abs().max())
+    ga, gb = torch.randn(n, generator=g, device=dev), torch.randn(n * 12, generator=g, device=dev)
+    ref = [torch.zeros(L.grid_bricked_elems(G, C), device=dev) for C in (1, 12)]
+    fl = [torch.zeros(L.grid_num_bricks(G), dtype=torch.uint8, device=dev) for _ in range(6)]
+    L.sample_grid_bwd2(ga, 1, ref[0], fl[0], gb, 12, ref[1], fl[1], gd, xyz, None, n, None)
+    up = _off_by(gb, sr)
+    one = _off_by(torch.zeros_like(ref[1]), sg)
+    L.sample_grid_bwd(up, gd, 12, xyz, None, n, None, one, fl[2])
+    pair = [torch.zeros_like(ref[0]), _off_by(torch.zeros_like(ref[1]), sg)]
+    L.sample_grid_bwd2(ga, 1, pair[0], fl[3], up, 12, pair[1], fl[4], gd, xyz, None, n, None)
+    for r, x in ((ref[1], one), (ref[0], pair[0]), (ref[1], pair[1])):
+        assert float((x - r).abs().max()) <= 1e-5 * float(r.abs().max())
+    for f in fl[1:5]:
+        assert torch.equal(f, fl[0])
+
+
 @pytest.mark.parametrize("shift", [0, 1], ids=["aligned", "unaligned"])
 @pytest.mark.parametrize("R", [1, 31, 1023, 1024, 1025, 8192, 8193, 152 * 1024 + 1, 400_001])
 def test_count_scan_blocks(L, R, shift):

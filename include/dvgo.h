@@ -35,8 +35,9 @@
  *    g[((z*Gy + y)*Gx + x)*C + c].
  *  - Buffers need their element type's own alignment and no more, except
  *    where a call states a rule (then checked on the host).  Trilinear
- *    queries of 12 channels and their adjoints are faster with rows and
- *    grids that start on 16-byte boundaries (BF16 grids: 8-byte).
+ *    queries of 12 channels, their adjoints and the TV gradient are faster
+ *    with rows and grids that start on 16-byte boundaries (BF16 grids:
+ *    8-byte).
  *
  * Which calls are the operations of the method, and which are fusions:
  *  - The operations (one call each, each the plain form of one step):

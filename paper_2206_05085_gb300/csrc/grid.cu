@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(512) mask_update_kernel(const void* __restrict
 // warp covers 32 consecutive voxels (contiguous memory) and the +-x/y/z
 // neighbours of most voxels sit in the same or an adjacent warp's lines.
 // Each thread handles all channels of its voxel with 128-bit loads when C % 4
-// == 0.  Neighbours are summed in the order -x, +x, -y, +y, -z, +z.
+// == 0 and the buffers are aligned for them, else one by one.  Neighbours are summed in the order -x, +x, -y, +y, -z, +z.
 __device__ __forceinline__ int compact3(uint32_t v) {
   return (int)((v & 1u) | ((v >> 2) & 2u) | ((v >> 4) & 4u));
 }
@@ -580,7 +580,7 @@ __device__ __forceinline__ void tv_neighbours(const BrickGeom& g, int64_t b, int
 
 // TV gradient of one voxel (thread t of brick b) of one grid.
 template <bool kBF16>
-__device__ __forceinline__ void tv_voxel(const void* __restrict__ grid, int C, float scale, float delta,
+__device__ __forceinline__ void tv_voxel(const void* __restrict__ grid, int C, bool vec, float scale, float delta,
                                          int dense_mode, float* __restrict__ g_grid, int64_t b, int t,
                                          const TvNbr& q) {
   const int64_t self = b * kBrickVox + t;
@@ -588,7 +588,7 @@ __device__ __forceinline__ void tv_voxel(const void* __restrict__ grid, int C, f
 #pragma unroll
   for (int d = 0; d < 6; ++d) nbr[d] = self + q.off[d];
   const bool* has = q.has;
-  if (C % 4 == 0) {
+  if (vec) {
     // sparse mode: a voxel whose data gradient is zero in every channel gets
     // no TV gradient, so its value and neighbours are not loaded at all
     if (!dense_mode) {
@@ -651,6 +651,7 @@ struct TvGridArgs {
   float scale;
   int C;
   int bf16;
+  int vec;   // C % 4 == 0 and buffers that four channels can be read from at once
 };
 struct TvMulti {
   TvGridArgs a[kMaxMulti];
@@ -680,9 +681,9 @@ __global__ void __launch_bounds__(512, 2) tv_kernel(TvMulti M, BrickGeom g, floa
       if (dense_mode && A.touched && t == 0) A.touched[b] = 1;
       if (!inside) continue;
       if (A.bf16)
-        tv_voxel<true>(A.grid, A.C, A.scale, delta, dense_mode, A.g_grid, b, t, q);
+        tv_voxel<true>(A.grid, A.C, A.vec, A.scale, delta, dense_mode, A.g_grid, b, t, q);
       else
-        tv_voxel<false>(A.grid, A.C, A.scale, delta, dense_mode, A.g_grid, b, t, q);
+        tv_voxel<false>(A.grid, A.C, A.vec, A.scale, delta, dense_mode, A.g_grid, b, t, q);
     }
   }
 }
@@ -1393,14 +1394,16 @@ extern "C" int dvgo_tv_add_grad_multi(const dvgo_tv_grid* grids, int32_t count, 
     const dvgo_tv_grid& q = grids[i];
     DVGO_CHECK_ARG(q.grid && q.g_grid && q.C >= 1 && (q.dtype == DVGO_F32 || q.dtype == DVGO_BF16));
     M.a[i] = TvGridArgs{q.grid, q.g_grid, q.touched, (float)((double)q.weight * 2.0 / (N * q.C)), q.C,
-                        q.dtype == DVGO_BF16 ? 1 : 0};
+                        q.dtype == DVGO_BF16 ? 1 : 0,
+                        q.C % 4 == 0 && (uintptr_t)q.g_grid % 16 == 0 &&
+                            (uintptr_t)q.grid % (q.dtype == DVGO_BF16 ? 8 : 16) == 0};
   }
   const bool use_list = !dense_mode && brick_list && brick_count;
   // a density and a feature grid (either order) over the list: the paired kernel
   if (use_list && count == 2 && M.a[0].bf16 == M.a[1].bf16 && M.a[0].C * M.a[1].C == 12 &&
       (M.a[0].C == 1 || M.a[1].C == 1)) {
     const TvGridArgs &D = M.a[M.a[0].C == 1 ? 0 : 1], &F = M.a[M.a[0].C == 1 ? 1 : 0];
-    if ((uintptr_t)F.g_grid % 16 == 0 && (uintptr_t)D.g_grid % 8 == 0 && (uintptr_t)F.grid % (F.bf16 ? 8 : 16) == 0) {
+    if (F.vec && (uintptr_t)D.g_grid % 8 == 0) {
       const int blocks = (int)std::min<int64_t>(g.num_bricks(), (int64_t)kNumSMs * 4);
       if (F.bf16)
         tv_pair_kernel<true><<<blocks, 32 * kTvWarps, 0, as_stream(stream)>>>(D, F, g, delta, brick_list, brick_count);

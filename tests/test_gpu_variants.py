@@ -375,6 +375,39 @@ def test_query12_off_alignment(L, bf16, which):
         assert torch.equal(f, fl[0])
 
 
+@pytest.mark.parametrize("which", ["grid", "gradient", "both"])
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("dense", [False, True])
+def test_tv_off_alignment(L, dense, bf16, which):
+    """TV of grids and gradients that start one element past a 16-byte boundary
+    (one channel at a time) against the aligned buffers: the same arithmetic per
+    entry, so the same bits; single, and paired with a density grid over the
+    brick list."""
+    dev, G = "cuda", (19, 23, 10)
+    nb = L.grid_num_bricks(G)
+    g = torch.Generator(device=dev).manual_seed(2)
+    dt, tdt = (L.BF16, torch.bfloat16) if bf16 else (L.F32, torch.float32)
+    sp, sg = int(which != "gradient"), int(which != "grid")
+    flags = (torch.rand(nb, generator=g, device=dev) < 0.7).to(torch.uint8)
+    flags[0] = 1
+    lst, cnt = torch.empty(nb, dtype=torch.int32, device=dev), torch.zeros(1, dtype=torch.int32, device=dev)
+    L.touched_compact(flags, nb, lst, cnt)
+    p = {C: torch.randn(nb * 512 * C, generator=g, device=dev).to(tdt) for C in (1, 4, 12)}
+    up = {C: torch.randn(nb * 512 * C, generator=g, device=dev)
+          * (torch.rand(nb * 512 * C, generator=g, device=dev) < 0.4) for C in (1, 4, 12)}
+    for C in (4, 12):
+        want, got = up[C].clone(), _off_by(up[C], sg)
+        L.tv_add_grad(p[C], dt, G, C, 1e-3, 0.5, dense, flags.clone(), want)
+        L.tv_add_grad(_off_by(p[C], sp), dt, G, C, 1e-3, 0.5, dense, flags.clone(), got)
+        assert torch.equal(got, want) and not torch.equal(want, up[C])
+    want = [up[1].clone(), up[12].clone()]
+    got = [_off_by(up[1], sg), _off_by(up[12], sg)]
+    for gr, off in ((want, 0), (got, 1)):
+        L.tv_add_grad_multi([(_off_by(p[C], off * sp), dt, C, 1e-3, flags.clone(), x) for C, x in zip((1, 12), gr)],
+                            G, 0.5, dense, None if dense else lst, None if dense else cnt)
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
 @pytest.mark.parametrize("shift", [0, 1], ids=["aligned", "unaligned"])
 @pytest.mark.parametrize("R", [1, 31, 1023, 1024, 1025, 8192, 8193, 152 * 1024 + 1, 400_001])
 def test_count_scan_blocks(L, R, shift):

@@ -913,6 +913,9 @@ __global__ void __launch_bounds__(256) adam_blocks_kernel(float* __restrict__ p,
   }
 }
 
+constexpr int kAdamWarps = 8, kAdamPerSM = 4;
+constexpr int kAdamGroups = 192;   // float4 groups a warp takes at once (a feature brick: eight such pieces)
+
 struct AdamArray {
   float* p;
   uint16_t* shadow;
@@ -924,6 +927,8 @@ struct AdamArray {
   int64_t block_elems;
   const int32_t* list;     // flagged blocks (or NULL: every block)
   const int32_t* list_n;
+  int64_t blocks;          // ceil(n / block_elems)
+  uint32_t groups;         // float4 groups of a block (of the array, if that is less)
   AdamArgs a;
 };
 struct AdamMulti {
@@ -932,88 +937,116 @@ struct AdamMulti {
   const int64_t* step;   // if set: t on the device, bias corrections formed in the kernel
 };
 
-// Blocks of all arrays in one index space: array i owns the next
-// |list_i| (or ceil(n_i / block_elems_i)) indices.
-__global__ void __launch_bounds__(256) adam_multi_kernel(AdamMulti M, int zero_grad) {
-  // bias corrections of the device-side step count, formed once by step_increment_kernel
-  float corr[2] = {0.0f, 0.0f};
-  if (M.step) {
-    const float* c = reinterpret_cast<const float*>(M.step + 1);
-    corr[0] = c[0];
-    corr[1] = c[1];
+// Blocks of all arrays in one index space: array i owns the next |list_i| (or
+// ceil(n_i / block_elems_i)) indices, and the thread blocks take them in turn.
+// corr: the bias corrections of a device-side step count, formed once by
+// step_increment_kernel.
+__device__ __forceinline__ void adam_block(const AdamArray& A, int64_t at, const float corr[2], bool dev_step,
+                                           int zero_grad) {
+  const int64_t lb = A.list ? (int64_t)A.list[at] : at;
+  if (A.touched && A.touched[lb] == 0) return;
+  AdamArgs a = A.a;
+  if (dev_step) {
+    a.inv_c1 = corr[0];
+    a.inv_c2 = corr[1];
   }
+  adam_range(A.p, A.shadow, A.g, A.m, A.v, lb * A.block_elems, min((lb + 1) * A.block_elems, A.n), a, zero_grad);
+  if (A.touched && zero_grad) {
+    __syncthreads();
+    if (threadIdx.x == 0) A.touched[lb] = 0;
+  }
+}
+
+__device__ __forceinline__ void adam_each_block(const AdamMulti& M, const float corr[2], int zero_grad) {
   int64_t first[kMaxMulti + 1];
   first[0] = 0;
   for (int i = 0; i < M.count; ++i) {
     const AdamArray& A = M.x[i];
-    first[i + 1] = first[i] + (A.list ? (int64_t)*A.list_n : (A.n + A.block_elems - 1) / A.block_elems);
+    first[i + 1] = first[i] + (A.list ? (int64_t)*A.list_n : A.blocks);
   }
   for (int64_t b = blockIdx.x; b < first[M.count]; b += gridDim.x) {
     int i = 0;
     while (i + 1 < M.count && b >= first[i + 1]) ++i;
-    const AdamArray& A = M.x[i];
-    const int64_t lb = A.list ? (int64_t)A.list[b - first[i]] : b - first[i];
-    if (A.touched && A.touched[lb] == 0) continue;
-    AdamArgs a = A.a;
-    if (M.step) {
-      a.inv_c1 = corr[0];
-      a.inv_c2 = corr[1];
-    }
-    adam_range(A.p, A.shadow, A.g, A.m, A.v, lb * A.block_elems, min((lb + 1) * A.block_elems, A.n), a,
-               zero_grad);
-    if (A.touched && zero_grad) {
-      __syncthreads();
-      if (threadIdx.x == 0) A.touched[lb] = 0;
-    }
+    adam_block(M.x[i], b - first[i], corr, M.step != nullptr, zero_grad);
   }
 }
 
-// adam_multi_kernel for arrays that bring a list of their flagged blocks (or
-// have no flags).  Every thread block owns a contiguous share of each array's
-// list, and its warps take 192-group pieces of those blocks (a feature brick:
-// eight) on their own: only the gradient is read whole (six float4 per lane in
-// flight), the non-zero groups go into the warp's queue in shared memory, and
-// full warps of them are updated, so that neither the state of all-zero
-// groups (five sixths of a forward-facing stack's touched bricks, two thirds
-// of an unbounded scene's) is read nor lanes idle in the update.  The flags are
-// cleared at the end, after the block's last barrier.  What bounds it: HBM.
-// Measured against adam_multi_kernel: 385 -> 283 us on a 384 x 384 x 256 stack
-// (17 % of the listed bricks' entries non-zero), 502 -> 444 us on 320^3
-// contracted (35 %), 41 -> 43 us on 160^3 (57 %), 16 -> 21 us on 64^3 (68 %, half
-// a brick per warp).  Reading the next piece ahead (80 registers, 24 warps per
-// SM) or gradient and state together for dense bricks was slower.
-constexpr int kAdamWarps = 8, kAdamPerSM = 4;
-constexpr int kAdamGroups = 192;
-struct AdamQueue {
-  float4 g[kAdamGroups + 32];
-  uint32_t id[kAdamGroups + 32];   // float4 group of the array
-};
-
-__global__ void __launch_bounds__(32 * kAdamWarps, kAdamPerSM) adam_list_kernel(AdamMulti M, int zero_grad) {
-  __shared__ AdamQueue queues[kAdamWarps];
-  __shared__ int64_t first[kMaxMulti];        // this thread block's share of each array's blocks
-  __shared__ int64_t count[kMaxMulti];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned below = (1u << lane) - 1u;
-  AdamQueue& q = queues[warp];
-  if (threadIdx.x < M.count) {
-    const AdamArray& A = M.x[threadIdx.x];
-    const int64_t nb = A.list ? (int64_t)*A.list_n : (A.n + A.block_elems - 1) / A.block_elems;
-    first[threadIdx.x] = nb * blockIdx.x / gridDim.x;
-    count[threadIdx.x] = nb * (blockIdx.x + 1) / gridDim.x - first[threadIdx.x];
-  }
-  float corr[2] = {0.0f, 0.0f};
+__device__ __forceinline__ void adam_corrections(const AdamMulti& M, float corr[2]) {
+  corr[0] = corr[1] = 0.0f;
   if (M.step) {
     const float* c = reinterpret_cast<const float*>(M.step + 1);
     corr[0] = c[0];
     corr[1] = c[1];
   }
+}
+
+__global__ void __launch_bounds__(256) adam_multi_kernel(const __grid_constant__ AdamMulti M, int zero_grad) {
+  float corr[2];
+  adam_corrections(M, corr);
+  adam_each_block(M, corr, zero_grad);
+}
+
+// adam_multi_kernel for arrays that bring a list of their flagged blocks (or
+// have no flags).  Every thread block owns a contiguous share of each array's
+// list, and its warps take kAdamGroups-group pieces of those blocks on their
+// own: only the gradient is read whole (six float4 per lane in flight), the
+// non-zero groups' indices go into the warp's queue in shared memory, and full
+// warps of them are updated, so that neither the state of all-zero groups (five
+// sixths of a forward-facing stack's touched bricks, two thirds of an unbounded
+// scene's) is read nor lanes idle in the update.  The flags are cleared at the
+// end, after the block's last barrier.  What bounds it: HBM.  Measured, after
+// the TV pass of a step, adam_multi_kernel and this form: 367 and 263 us on a
+// 384 x 384 x 256 stack (18,268 listed bricks, 16 % of their groups non-zero),
+// 391 and 325 us on 320^3 contracted (17,437; 27 %), 83 and 73 us on 160^3
+// contracted (2972), 47.3 and 47.9 us on 160^3 bounded (1497; 60 %), 86.5 and
+// 82 us on 200^3 bounded (2703).
+//
+// A list that gives no warp more than one piece (about 560 bricks of both
+// grids; the lists' lengths are on the device) is left to adam_multi_kernel's
+// loop: gradient and state loaded together, a whole thread block on a brick.
+// There the queue's two round trips and one piece per warp are what is waited
+// for: 484 bricks of 100^3 23.1 us in adam_multi_kernel, 26.6 with the queue,
+// 23.3-24.4 so.  (889 of 128^3 31.0, 33.4 and 33.0; but 887 of a 128 x 128 x 64
+// stack 27.2, 26.0 and 28.9.)  Grids that have no more bricks than that go to
+// adam_multi_kernel itself (498 of 64^3's 512: 23.1 us, 24.1 here).  The queue holds
+// indices only: with the gradients in it 36 KB a thread block left the L1 too
+// little room for the loads in flight (498 bricks 27.4, 1497 of 160^3 49.2 us).
+struct AdamQueue {
+  uint32_t id[kAdamGroups + 32];   // float4 groups of the array
+};
+
+__global__ void __launch_bounds__(32 * kAdamWarps, kAdamPerSM) adam_list_kernel(
+    const __grid_constant__ AdamMulti M, int zero_grad) {
+  __shared__ AdamQueue queues[kAdamWarps];
+  __shared__ uint32_t first[kMaxMulti];       // this thread block's share of each array's blocks
+  __shared__ uint32_t count[kMaxMulti];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned below = (1u << lane) - 1u;
+  AdamQueue& q = queues[warp];
+  float corr[2];
+  adam_corrections(M, corr);
+  const uint32_t blocks = min(gridDim.x, (uint32_t)(kNumSMs * kAdamPerSM));
+  int64_t work = 0;   // groups of all arrays' blocks
+  for (int i = 0; i < M.count; ++i) {
+    const AdamArray& A = M.x[i];
+    const uint32_t nb = A.list ? (uint32_t)*A.list_n : (uint32_t)A.blocks, each = nb / blocks, left = nb % blocks;
+    work += (int64_t)nb * A.groups;
+    if (threadIdx.x == 0) {
+      first[i] = each * blockIdx.x + min(blockIdx.x, left);
+      count[i] = each + (blockIdx.x < left ? 1u : 0u);
+    }
+  }
+  if (work <= (int64_t)kAdamGroups * kAdamWarps * blocks) {   // at most one piece a warp
+    adam_each_block(M, corr, zero_grad);
+    return;
+  }
+  if (blockIdx.x >= blocks) return;
   __syncthreads();
-  int64_t u = warp;   // the warp's next piece, counted within array ai
+  uint32_t u = warp;   // the warp's next piece, counted within array ai
   for (int ai = 0; ai < M.count; ++ai) {
     const AdamArray& A = M.x[ai];
-    const int pieces = (int)((A.block_elems / 4 + kAdamGroups - 1) / kAdamGroups);
-    const int64_t total = count[ai] * pieces;
+    const uint32_t pieces = (A.groups + kAdamGroups - 1) / kAdamGroups;
+    const uint32_t total = count[ai] * pieces;
     if (u >= total) {
       u -= total;
       continue;
@@ -1028,16 +1061,17 @@ __global__ void __launch_bounds__(32 * kAdamWarps, kAdamPerSM) adam_list_kernel(
     int n = 0;   // queued groups
     auto update = [&](int at) {
       const int64_t i = 4 * (int64_t)q.id[at];
+      const float4 gg = *reinterpret_cast<const float4*>(g + i);
       const float4 pp = *reinterpret_cast<const float4*>(p + i);
       const float4 mm = *reinterpret_cast<const float4*>(m + i);
       const float4 vv = *reinterpret_cast<const float4*>(v + i);
-      adam_group(p, shadow, g, m, v, i, q.g[at], pp, mm, vv, a, zero_grad);
+      adam_group(p, shadow, g, m, v, i, gg, pp, mm, vv, a, zero_grad);
     };
     for (; u < total; u += kAdamWarps) {
-      const int64_t b = first[ai] + u / pieces;
-      const int64_t lb = A.list ? (int64_t)__ldg(A.list + b) : b;
+      const uint32_t b = u / pieces, piece = u - b * pieces;
+      const int64_t lb = A.list ? (int64_t)__ldg(A.list + first[ai] + b) : (int64_t)(first[ai] + b);
       const uint8_t flag = A.touched ? A.touched[lb] : (uint8_t)1;
-      const int64_t c0 = lb * A.block_elems + 4 * (int64_t)kAdamGroups * (u % pieces);
+      const int64_t c0 = lb * A.block_elems + 4 * (int64_t)kAdamGroups * piece;
       const int64_t stop = min(min((lb + 1) * A.block_elems, A.n), c0 + 4 * kAdamGroups);
       float4 gg[kAdamGroups / 32];
 #pragma unroll
@@ -1053,7 +1087,6 @@ __global__ void __launch_bounds__(32 * kAdamWarps, kAdamPerSM) adam_list_kernel(
         const unsigned bal = __ballot_sync(0xffffffffu, nz);
         if (nz) {
           const int at = n + __popc(bal & below);
-          q.g[at] = gg[k];
           q.id[at] = (uint32_t)(c0 / 4) + lane + 32 * k;
         }
         n += __popc(bal);
@@ -1061,14 +1094,16 @@ __global__ void __launch_bounds__(32 * kAdamWarps, kAdamPerSM) adam_list_kernel(
       __syncwarp();
       for (; n >= 64; n -= 64) {
         const int64_t i = 4 * (int64_t)q.id[n - 64 + lane], j = 4 * (int64_t)q.id[n - 32 + lane];
+        const float4 g0 = *reinterpret_cast<const float4*>(g + i);
+        const float4 g1 = *reinterpret_cast<const float4*>(g + j);
         const float4 p0 = *reinterpret_cast<const float4*>(p + i);
         const float4 m0 = *reinterpret_cast<const float4*>(m + i);
         const float4 v0 = *reinterpret_cast<const float4*>(v + i);
         const float4 p1 = *reinterpret_cast<const float4*>(p + j);
         const float4 m1 = *reinterpret_cast<const float4*>(m + j);
         const float4 v1 = *reinterpret_cast<const float4*>(v + j);
-        adam_group(p, shadow, g, m, v, i, q.g[n - 64 + lane], p0, m0, v0, a, zero_grad);
-        adam_group(p, shadow, g, m, v, j, q.g[n - 32 + lane], p1, m1, v1, a, zero_grad);
+        adam_group(p, shadow, g, m, v, i, g0, p0, m0, v0, a, zero_grad);
+        adam_group(p, shadow, g, m, v, j, g1, p1, m1, v1, a, zero_grad);
       }
       if (n >= 32) {
         n -= 32;
@@ -1093,7 +1128,7 @@ __global__ void __launch_bounds__(32 * kAdamWarps, kAdamPerSM) adam_list_kernel(
   for (int ai = 0; ai < M.count; ++ai) {
     const AdamArray& A = M.x[ai];
     if (!A.touched) continue;
-    for (int64_t i = threadIdx.x; i < count[ai]; i += blockDim.x) A.touched[A.list[first[ai] + i]] = 0;
+    for (uint32_t i = threadIdx.x; i < count[ai]; i += blockDim.x) A.touched[A.list[first[ai] + i]] = 0;
   }
 }
 
@@ -1523,7 +1558,7 @@ static int adam_multi(const dvgo_adam_param* params, int32_t count, float beta1,
   AdamMulti M{};
   M.count = 0;
   M.step = step_dev;
-  int64_t total = 0;
+  int64_t total = 0, work = 0;   // blocks of all arrays, and their groups
   bool lists = false;
   const float inv_c1 = (float)(1.0 / (1.0 - pow((double)beta1, (double)step)));
   const float inv_c2 = (float)(1.0 / (1.0 - pow((double)beta2, (double)step)));
@@ -1541,18 +1576,21 @@ static int adam_multi(const dvgo_adam_param* params, int32_t count, float beta1,
     AdamArray& A = M.x[M.count++];
     A = AdamArray{q.p, q.p_shadow, q.g, q.m, q.v, q.n, q.touched, be,
                   use_list ? q.block_list : nullptr, use_list ? q.block_count : nullptr,
+                  (q.n + be - 1) / be, (uint32_t)(std::min(be, (q.n + 3) / 4 * 4) / 4),
                   AdamArgs{q.lr, beta1, beta2, eps, inv_c1, inv_c2}};
-    total += (q.n + be - 1) / be;
+    total += A.blocks;
+    work += A.blocks * A.groups;
   }
   if (M.count == 0) return DVGO_OK;
   // every flagged array with its list (and 32-bit group indices): the list
-  // kernel.  Else with lists the block count is on the device: persistent
-  // blocks; without, one block per block of entries
-  bool list_form = lists;
+  // kernel (short lists use all of its thread blocks, others half), unless
+  // even whole lists would be short ones.  Else with lists the block count is
+  // on the device: persistent blocks; without, one block per block of entries
+  bool list_form = lists && work > (int64_t)kAdamGroups * kAdamWarps * std::min<int64_t>(total, kNumSMs * kAdamPerSM);
   for (int i = 0; i < M.count; ++i)
     list_form = list_form && (!M.x[i].touched || M.x[i].list) && M.x[i].n < ((int64_t)1 << 34);
   if (list_form) {
-    adam_list_kernel<<<(int)std::min<int64_t>(total, (int64_t)kNumSMs * kAdamPerSM), 32 * kAdamWarps, 0,
+    adam_list_kernel<<<(int)std::min<int64_t>(total, (int64_t)kNumSMs * 2 * kAdamPerSM), 32 * kAdamWarps, 0,
                        as_stream(stream)>>>(M, zero_grad);
     return launch_status();
   }

@@ -161,6 +161,39 @@ def test_adam_list_against_single_arrays(L, n_flat, density):
     assert int(f[0].sum()) == 0 and int(f[1].sum()) == 0
 
 
+@pytest.mark.parametrize("listed", [1, 557, 561, 562, 565, 2000, 5000])   # both sides of one piece a warp; many pieces
+@pytest.mark.parametrize("density", [0.03, 0.5, 1.0])
+@pytest.mark.parametrize("zero_grad", [True, False])
+def test_adam_list_lengths(L, listed, density, zero_grad):
+    """The list kernel at lengths of either of its loops, with whole bricks and
+    single groups of zero gradients, against the call per array: the same bits,
+    flags cleared (or, without zero_grad, gradients and flags kept)."""
+    nb, dev = 5003, "cuda"
+    g = torch.Generator(device=dev).manual_seed(listed)
+    flags = torch.zeros(nb, dtype=torch.uint8, device=dev)
+    flags[torch.randperm(nb, generator=g, device=dev)[:listed]] = 1
+    lst, cnt = torch.empty(nb, dtype=torch.int32, device=dev), torch.zeros(1, dtype=torch.int32, device=dev)
+    L.touched_compact(flags, nb, lst, cnt)
+
+    def state(C):
+        p, m = (torch.randn(nb * 512 * C, generator=g, device=dev) for _ in range(2))
+        grad = torch.randn(nb * 512 * C, generator=g, device=dev)
+        keep = (torch.rand(nb * 128 * C, generator=g, device=dev) < density).repeat_interleave(4)
+        keep &= (torch.rand(nb, generator=g, device=dev) < 0.9).repeat_interleave(512 * C)
+        return [p, grad * keep, m, m.abs()]
+    sets = [state(1), state(12)]
+    ref = [[x.clone() for x in s] for s in sets]
+    f = [flags.clone() for _ in range(4)]
+    L.adam_step_multi([(s[0], None, *s[1:], s[0].numel(), f[i], 512 * (1, 12)[i], 0.1, lst, cnt)
+                       for i, s in enumerate(sets)], 0.9, 0.99, 1e-15, 3, zero_grad)
+    for i, s in enumerate(ref):
+        L.adam_step(s[0], None, *s[1:], s[0].numel(), f[2 + i], 512 * (1, 12)[i], 0.1, 0.9, 0.99, 1e-15, 3, zero_grad)
+    for a, b in zip(sets, ref):
+        for x, y in zip(a, b):
+            assert torch.equal(x, y)
+    assert all(torch.equal(x, torch.zeros_like(flags) if zero_grad else flags) for x in f)
+
+
 @pytest.mark.parametrize("G", [(61, 47, 53), (8, 8, 8), (9, 16, 17)])
 @pytest.mark.parametrize("bf16", [False, True])
 def test_tv_pair_against_single_grids(L, G, bf16):

@@ -525,9 +525,10 @@ __global__ void __launch_bounds__(32 * kCkpt) contracted_fill_kernel(
 // counts and scans them 1024 a pass (one a thread); what lies before them it
 // adds up for itself, so the blocks wait for nothing.  Even the last one reads
 // each count once, as one block alone would, and the offsets, most of the
-// traffic, are written by all.  Bound by the latency of a pass.  Measured, one
-// block alone with 8192 counts a pass and this form: 7.3 and 3.8 us for 16,384
-// counts, 4.1 and 3.2 us for 8192, 3.4 us both for 4099.
+// traffic, are written by all.  Bound by the latency of a pass.  Measured with
+// the live list's fill of empty rays, one block alone with 8192 counts a pass
+// and this form: 9.2 and 5.6 us for 16,384 counts, 5.9 and 4.7 us for 8192, 1580
+// and 199 us for 4.2e6.
 __host__ __device__ constexpr int64_t scan_chunk(int64_t n, int blocks) {
   return ((n + blocks - 1) / blocks + 1023) / 1024 * 1024;
 }
@@ -585,6 +586,73 @@ __global__ void __launch_bounds__(1024) scan_counts_kernel(const int32_t* __rest
     off[n] = carry;
     if (total_out) *total_out = carry;
   }
+}
+
+// The same for n <= kScanSmall in one block: eight consecutive counts a thread,
+// ceil(n / 8) threads (whole warps), one barrier.  Bound by its latency (one
+// load, two warp scans).  Where the line lies: the live list's scan and fill of
+// empty rays take 3.0 us so and 4.0 us with scan_counts_kernel for 256 counts,
+// 3.5 and 4.3 for 2048, 4.2 and 4.6 for 4096, but 5.0 and 4.5 for 6144.
+constexpr int64_t kScanSmall = 4096;
+static_assert(kScanSmall <= 8 * 1024, "one block of eight counts a thread");
+
+__global__ void __launch_bounds__(1024) scan_small_kernel(const int32_t* __restrict__ counts, int n,
+                                                          int64_t* __restrict__ off,
+                                                          int64_t* __restrict__ total_out) {
+  __shared__ int64_t warp_tot[32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, i0 = 8 * threadIdx.x;
+  int32_t c[8];
+  if ((reinterpret_cast<uintptr_t>(counts) & 15u) == 0 && i0 + 8 <= n) {
+    const int4 a = __ldg(reinterpret_cast<const int4*>(counts + i0));
+    const int4 b = __ldg(reinterpret_cast<const int4*>(counts + i0 + 4));
+    c[0] = a.x; c[1] = a.y; c[2] = a.z; c[3] = a.w;
+    c[4] = b.x; c[5] = b.y; c[6] = b.z; c[7] = b.w;
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) c[k] = i0 + k < n ? __ldg(counts + i0 + k) : 0;
+  }
+  int64_t loc[8], s = 0;   // sums of the thread's counts before each
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    loc[k] = s;
+    s += c[k];
+  }
+  int64_t incl = s;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) warp_tot[wid] = incl;
+  __syncthreads();
+  int64_t v = lane < (int)(blockDim.x >> 5) ? warp_tot[lane] : 0;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
+  }
+  const int64_t prev = __shfl_sync(0xffffffffu, v, wid > 0 ? wid - 1 : 0), total = __shfl_sync(0xffffffffu, v, 31);
+  const int64_t ex = (wid > 0 ? prev : 0) + incl - s;
+  if (i0 + 8 <= n && (reinterpret_cast<uintptr_t>(off) & 15u) == 0) {
+#pragma unroll
+    for (int k = 0; k < 8; k += 2)
+      *reinterpret_cast<longlong2*>(off + i0 + k) = make_longlong2(ex + loc[k], ex + loc[k + 1]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (i0 + k < n) off[i0 + k] = ex + loc[k];
+  }
+  if (threadIdx.x == 0) {
+    off[n] = total;
+    if (total_out) *total_out = total;
+  }
+}
+
+static void scan_counts(const int32_t* counts, int64_t n, int64_t* off, int64_t* total_out, cudaStream_t st) {
+  if (n <= kScanSmall)
+    scan_small_kernel<<<1, (int)(n + 255) / 256 * 32, 0, st>>>(counts, (int)n, off, total_out);
+  else
+    scan_counts_kernel<<<scan_blocks(n), 1024, 0, st>>>(counts, n, off, total_out);
 }
 
 // Live list: live_idx[live_off[r] + i] = ray_off[r] + i for i < seg_len[r].
@@ -707,12 +775,12 @@ extern "C" int dvgo_sample_rays(const float* rays_o, const float* rays_d, int64_
                          : nullptr;
     if (smp->mode == 0) {
       bbox_count_kernel<false><<<g, block, 0, st>>>(A, rays_o, rays_d, R, mask, counts, bits);
-      scan_counts_kernel<<<scan_blocks(R), 1024, 0, st>>>(counts, R, ray_off, nullptr);
+      scan_counts(counts, R, ray_off, nullptr, st);
       bbox_fill_kernel<false><<<g, block, 0, st>>>(A, rays_o, rays_d, R, mask, bits, ray_off, xyz, ray_id,
                                                    step_k, s_mid, s_len);
     } else {
       bbox_count_kernel<true><<<g, block, 0, st>>>(A, rays_o, rays_d, R, mask, counts, bits);
-      scan_counts_kernel<<<scan_blocks(R), 1024, 0, st>>>(counts, R, ray_off, nullptr);
+      scan_counts(counts, R, ray_off, nullptr, st);
       bbox_fill_kernel<true><<<g, block, 0, st>>>(A, rays_o, rays_d, R, mask, bits, ray_off, xyz, ray_id,
                                                   step_k, s_mid, s_len);
     }
@@ -726,7 +794,7 @@ extern "C" int dvgo_sample_rays(const float* rays_o, const float* rays_d, int64_
     uint32_t* ckpt = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + counts_bytes(R));
     contracted_kernel<false><<<g, block, 0, st>>>(A, rays_o, rays_d, R, mask, counts, ckpt,
                                                   nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
-    scan_counts_kernel<<<scan_blocks(R), 1024, 0, st>>>(counts, R, ray_off, nullptr);
+    scan_counts(counts, R, ray_off, nullptr, st);
     contracted_fill_kernel<<<(int)ceil_div(R, 32), 32 * kCkpt, 0, st>>>(A, rays_d, R, mask, ckpt, ray_off,
                                                                         xyz, ray_id, step_k, s_mid, s_len);
   }
@@ -754,7 +822,7 @@ extern "C" int dvgo_live_samples_cull(const int64_t* ray_off, const int32_t* seg
                                                (size_t)((R + 1) * sizeof(int64_t) + 255) / 256 * 256);
   const int g = grid_for(R * 32, 256, 16);
   cull_kernel<false><<<g, 256, 0, st>>>(ray_off, seg_len, w, w_min, R, counts, nullptr, nullptr, nullptr, nullptr);
-  scan_counts_kernel<<<scan_blocks(R), 1024, 0, st>>>(counts, R, off, live_count);
+  scan_counts(counts, R, off, live_count, st);
   cull_kernel<true><<<g, 256, 0, st>>>(ray_off, seg_len, w, w_min, R, nullptr, off, live_idx, rgb, g_k0);
   return launch_status();
 }
@@ -770,7 +838,7 @@ extern "C" int dvgo_live_samples(const int64_t* ray_off, const int32_t* seg_len,
     return launch_status();
   }
   int64_t* live_off = reinterpret_cast<int64_t*>(ws);
-  scan_counts_kernel<<<scan_blocks(R), 1024, 0, st>>>(seg_len, R, live_off, live_count);
+  scan_counts(seg_len, R, live_off, live_count, st);
   live_fill_kernel<<<grid_for(R * 32, 256, 16), 256, 0, st>>>(ray_off, seg_len, R, live_off,
                                                               live_idx);
   return launch_status();
@@ -886,14 +954,14 @@ extern "C" int dvgo_sample_rays_noalloc(const float* rays_o, const float* rays_d
     const int block = 256;
     int g = grid_for(R * 32, block, 16);
     bbox_count_kernel<false><<<g, block, 0, st>>>(A, rays_o, rays_d, R, mask, counts, nullptr);
-    scan_counts_kernel<<<scan_blocks(R), 1024, 0, st>>>(counts, R, ray_off, nullptr);
+    scan_counts(counts, R, ray_off, nullptr, st);
     bbox_fill_kernel<false><<<g, block, 0, st>>>(A, rays_o, rays_d, R, mask, nullptr, ray_off, xyz,
                                                  ray_id, step_k, s_mid, s_len);
   } else if (smp->mode == 2) {
     const int block = 256;
     int g = grid_for(R * 32, block, 16);
     bbox_count_kernel<true><<<g, block, 0, st>>>(A, rays_o, rays_d, R, mask, counts, nullptr);
-    scan_counts_kernel<<<scan_blocks(R), 1024, 0, st>>>(counts, R, ray_off, nullptr);
+    scan_counts(counts, R, ray_off, nullptr, st);
     bbox_fill_kernel<true><<<g, block, 0, st>>>(A, rays_o, rays_d, R, mask, nullptr, ray_off, xyz,
                                                 ray_id, step_k, s_mid, s_len);
   } else {
@@ -903,7 +971,7 @@ extern "C" int dvgo_sample_rays_noalloc(const float* rays_o, const float* rays_d
     int g = (int)ceil_div(R, block);
     contracted_kernel<false><<<g, block, 0, st>>>(A, rays_o, rays_d, R, mask, counts, nullptr,
                                                   nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
-    scan_counts_kernel<<<scan_blocks(R), 1024, 0, st>>>(counts, R, ray_off, nullptr);
+    scan_counts(counts, R, ray_off, nullptr, st);
     contracted_kernel<true><<<g, block, 0, st>>>(A, rays_o, rays_d, R, mask, nullptr, nullptr, ray_off, xyz,
                                                  ray_id, step_k, s_mid, s_len);
   }

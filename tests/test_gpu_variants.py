@@ -463,6 +463,14 @@ def test_count_scan_blocks(L, R, shift):
     assert np.array_equal(idx.cpu().numpy()[:n], want)
 
 
+@pytest.mark.parametrize("shift", [0, 1], ids=["aligned", "unaligned"])
+@pytest.mark.parametrize("R", [7, 8, 9, 255, 256, 257, 4095, 4096, 4097])
+def test_count_scan_small(L, R, shift):
+    """The one-block scan: remainders of a thread's eight counts, a last thread
+    of a warp, and both sides of its largest length."""
+    test_count_scan_blocks(L, R, shift)
+
+
 @pytest.mark.parametrize("steps", [1, 7, 8, 61, 130, 512])
 @pytest.mark.parametrize("R", [1, 31, 33, 300])
 def test_contracted_fill_groups(L, R, steps):

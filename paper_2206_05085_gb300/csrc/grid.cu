@@ -246,7 +246,7 @@ struct ScatterStage {
   uint8_t rep[32];
 };
 
-template <bool kA, bool kB>
+template <bool kA, bool kB, int kPer>
 __global__ void __launch_bounds__(256) scatter_merge_kernel(
     const float* __restrict__ g_a, float* __restrict__ grid_a, uint8_t* __restrict__ touched_a,
     const float* __restrict__ g_b, float* __restrict__ grid_b, uint8_t* __restrict__ touched_b, TriArgs T,
@@ -260,9 +260,9 @@ __global__ void __launch_bounds__(256) scatter_merge_kernel(
   // over half a sample per voxel: the density's reductions are spread between
   // the features' (bursts of them meet in the few sectors they have)
   const bool crowded = 2 * n > (int64_t)T.g.G[0] * T.g.G[1] * T.g.G[2];
-  for (int64_t j0 = warp0 * 32; j0 < n; j0 += nwarps * 32) {
+  for (int64_t j0 = warp0 * kPer; j0 < n; j0 += nwarps * kPer) {
     const int64_t j = j0 + lane;
-    const bool valid = j < n;
+    const bool valid = lane < kPer && j < n;
     Corners c;
     float ga = 0.0f, gb[12];
 #pragma unroll
@@ -300,18 +300,15 @@ __global__ void __launch_bounds__(256) scatter_merge_kernel(
     const unsigned abs_mask = __ballot_sync(0xffffffffu, absorbed);
     if constexpr (!kB) {
       // one channel: the lane issues its cell's eight reductions
+      const bool pair = lane < 31 && ((abs_mask >> (lane + 1)) & 1u);
       float wn[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) wn[k] = __shfl_down_sync(0xffffffffu, c.w[k], 1);
-      const float gan = __shfl_down_sync(0xffffffffu, ga, 1);
+      float gan = __shfl_down_sync(0xffffffffu, ga, 1);
+      if (!pair) gan = 0.0f;   // (the weights are finite; an infinite gradient times 0 would not be)
       if (!valid || absorbed) continue;
-      const bool pair = lane < 31 && ((abs_mask >> (lane + 1)) & 1u);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {   // (a neighbour that is not merged is left out, not weighted by 0: it may be infinite)
-        float v = c.w[k] * ga;
-        if (pair) v = fmaf(wn[k], gan, v);
-        atomicAdd(grid_a + c.slot[k], v);
-      }
+      for (int k = 0; k < 8; ++k) atomicAdd(grid_a + c.slot[k], fmaf(wn[k], gan, c.w[k] * ga));
       mark_touched(touched_a, T, c);
     } else {
       __syncwarp();   // the last step's rows have been read
@@ -1385,6 +1382,29 @@ extern "C" int dvgo_sample_grid_fwd(const void* grid, int dtype, const dvgo_grid
   return launch_status();
 }
 
+// Up to kScatterFew samples a warp takes eight list positions instead of 32: there
+// the chip is far from full, and a warp's merged samples going out one after the
+// other are what is waited for.  Measured on samples along rays of 160^3, eight
+// and 32 positions (a lane per sample and float4, before the merged form): 12
+// channels, 256 samples 3.0 and 4.2 us (4.8), 4096 samples 3.2 and 4.4 (5.2);
+// both grids, 32 samples 2.9 and 3.2 (2.7), 4096 samples 3.7 and 5.1 us (5.5).
+// Beyond, the reductions of more warps get in each other's way: 16,384 random
+// points of 64^3, 12 channels, 10.4 and 7.4 us.  (A single sample, 2.1 us, and
+// up to 130,000 points in no order, one channel, remain 0.3 us and 3-9 % above
+// the unmerged form's times: the look for neighbours in one cell.)
+constexpr int64_t kScatterFew = 4096;
+template <bool kA, bool kB>
+static void scatter_merge(const float* g_a, float* grid_a, uint8_t* touched_a, const float* g_b, float* grid_b,
+                          uint8_t* touched_b, const TriArgs& T, const float* xyz, const int32_t* idx, int64_t n_cap,
+                          const int64_t* n_dev, cudaStream_t st) {
+  if (n_cap <= kScatterFew)
+    scatter_merge_kernel<kA, kB, 8><<<grid_for(4 * n_cap, 256, 16), 256, 0, st>>>(
+        g_a, grid_a, touched_a, g_b, grid_b, touched_b, T, xyz, idx, n_cap, n_dev);
+  else
+    scatter_merge_kernel<kA, kB, 32><<<grid_for(n_cap, 256, 16), 256, 0, st>>>(
+        g_a, grid_a, touched_a, g_b, grid_b, touched_b, T, xyz, idx, n_cap, n_dev);
+}
+
 extern "C" int dvgo_sample_grid_bwd(const float* g_out, const dvgo_grid_desc* gd, int32_t C,
                                     const float* xyz, const int32_t* idx, int64_t n_cap,
                                     const int64_t* n_dev, float* g_grid, uint8_t* touched,
@@ -1395,15 +1415,13 @@ extern "C" int dvgo_sample_grid_bwd(const float* g_out, const dvgo_grid_desc* gd
   TriArgs T;
   DVGO_CHECK_ARG(make_tri(T, gd));
   cudaStream_t st = as_stream(stream);
-  const int block = 256;
-  int g = grid_for(n_cap, block, 16);
   if (C == 1)
-    scatter_merge_kernel<true, false><<<g, block, 0, st>>>(g_out, g_grid, touched, nullptr, nullptr, nullptr, T, xyz,
-                                                           idx, n_cap, n_dev);
+    scatter_merge<true, false>(g_out, g_grid, touched, nullptr, nullptr, nullptr, T, xyz, idx, n_cap, n_dev, st);
   else if (C == 12 && (uintptr_t)g_out % 16 == 0 && (uintptr_t)g_grid % 16 == 0)   // rows and voxels by float4
-    scatter_merge_kernel<false, true><<<g, block, 0, st>>>(nullptr, nullptr, nullptr, g_out, g_grid, touched, T, xyz,
-                                                           idx, n_cap, n_dev);
-  else scatter_bwd_generic_kernel<<<g, block, 0, st>>>(g_out, T, C, xyz, idx, n_cap, n_dev, g_grid, touched);
+    scatter_merge<false, true>(nullptr, nullptr, nullptr, g_out, g_grid, touched, T, xyz, idx, n_cap, n_dev, st);
+  else
+    scatter_bwd_generic_kernel<<<grid_for(n_cap, 256, 16), 256, 0, st>>>(g_out, T, C, xyz, idx, n_cap, n_dev, g_grid,
+                                                                        touched);
   return launch_status();
 }
 
@@ -1503,8 +1521,8 @@ extern "C" int dvgo_sample_grid_bwd2(const float* g_out_a, int32_t C_a, float* g
     TriArgs T;
     DVGO_CHECK_ARG(make_tri(T, gd));
     cudaStream_t st = as_stream(stream);
-    scatter_merge_kernel<true, true><<<grid_for(n_cap, 256, 16), 256, 0, st>>>(
-        g_out_a, g_grid_a, touched_a, g_out_b, g_grid_b, touched_b, T, xyz, idx, n_cap, n_dev);
+    scatter_merge<true, true>(g_out_a, g_grid_a, touched_a, g_out_b, g_grid_b, touched_b, T, xyz, idx, n_cap, n_dev,
+                              st);
     return launch_status();
   }
   int r = dvgo_sample_grid_bwd(g_out_a, gd, C_a, xyz, idx, n_cap, n_dev, g_grid_a, touched_a, stream);

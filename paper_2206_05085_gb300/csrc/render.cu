@@ -295,7 +295,10 @@ __device__ __forceinline__ int last_chunk_of(int n) { return n > 0 ? ((n - 1) & 
 // the last chunk's, which the caller starts before the sums over the ray).
 // Measured, the fused per-ray tail of a step with 8192 rays: 33.5 us with the
 // loads of a chunk at its start, 23.6 us ahead (160^3, 393,909 samples); 86
-// and 65 us (320^3 unbounded, 1.9e6 samples); 13.0 and 10.4 us (64^3).
+// and 65 us (320^3 unbounded, 1.9e6 samples); 13.0 and 10.4 us (64^3).  Many
+// rays of one chunk each gain nothing from it: 30,000 of at most 24 samples
+// 24.2 and 24.8 us (25.1 with all of the first chunk's loads repeated), the
+// adjoint alone 12.8 and 13.6 us.
 __device__ __forceinline__ void composite_distortion_bwd_ray(
     int lane, int64_t b, int n, int N, BwdSample next, float gc0, float gc1, float gc2, float Wt, float WMt,
     float g_L,
@@ -454,8 +457,12 @@ __global__ void __launch_bounds__(256) composite_distortion_fwd_kernel(
     }
     BwdSample first;
     if constexpr (kBwd) {
+      // (the forward's loads end with the last chunk's: only raw, T and the interval are new)
       const int k = last_chunk_of(n) + lane;
-      first.load(k >= 0 && k < n, b + k, w, bt.raw, bt.T, rgb, m, ds, bt.interval, bt.delta);
+      const bool valid = k >= 0 && k < n;
+      first = valid ? BwdSample{nw, nm, nd, __ldg(bt.raw + b + k), __ldg(bt.T + b + k), nc0, nc1, nc2,
+                                interval_of(bt.delta, bt.interval, b + k)}
+                    : BwdSample{};
     }
     a0 = warp_sum(a0);
     a1 = warp_sum(a1);

@@ -367,6 +367,67 @@ def test_scatter_merge_nonfinite_rows(L, form, bad):
         assert bool((diff <= 1e-5 * float(ref.abs().max())).all())     # (NaN compares false)
 
 
+@pytest.mark.parametrize("form", ["a", "b", "ab"])
+def test_scatter_merge_second_trip(L, form):
+    """More samples than the launch's warps take at once (2432 x 8 warps of 32):
+    a warp's rows in shared memory are written again.  Sums of at most some
+    hundred FP32 terms per voxel: 1e-5 of the largest entry; the flags are
+    exactly the bricks of the samples' cells."""
+    dev, n, G = "cuda", 650_001, (61, 70, 83)
+    g = torch.Generator(device=dev).manual_seed(6)
+    base = torch.rand(n // 2 + 1, 3, generator=g, device=dev) * 0.9 - 0.8     # a part of the grid
+    xyz = (base.repeat_interleave(2, 0)[:n] + 0.004 * torch.rand(n, 3, generator=g, device=dev)).contiguous()
+    ga, gb = torch.randn(n, generator=g, device=dev), torch.randn(n, 12, generator=g, device=dev)
+    gd = L.GridDesc.make(-1.0, 1.0, G)
+    out = [torch.zeros(L.grid_bricked_elems(G, C), device=dev) for C in (1, 12)]
+    fl = [torch.zeros(L.grid_num_bricks(G), dtype=torch.uint8, device=dev) for _ in range(2)]
+    if form == "ab":
+        L.sample_grid_bwd2(ga, 1, out[0], fl[0], gb, 12, out[1], fl[1], gd, xyz, None, n, None)
+    elif form == "a":
+        L.sample_grid_bwd(ga, gd, 1, xyz, None, n, None, out[0], fl[0])
+    else:
+        L.sample_grid_bwd(gb, gd, 12, xyz, None, n, None, out[1], fl[1])
+    dim = torch.tensor(G, device=dev)
+    u = (xyz.double() + 1) * 0.5 * (dim - 1)
+    i, nb = u.floor().long(), [(x + 7) // 8 for x in G]
+    f = u - i
+    want = torch.zeros(L.grid_num_bricks(G), dtype=torch.uint8, device=dev)
+    ref = {C: torch.zeros(G[2] * G[1] * G[0], C, dtype=torch.float64, device=dev) for C in (1, 12)}
+    for k in range(8):
+        c = i + torch.tensor([k & 1, (k >> 1) & 1, k >> 2], device=dev)
+        w = torch.where((c > i), f, 1 - f).prod(1, keepdim=True)
+        want[((c[:, 2] >> 3) * nb[1] + (c[:, 1] >> 3)) * nb[0] + (c[:, 0] >> 3)] = 1
+        for C, up in ((1, ga[:, None]), (12, gb)):
+            ref[C].index_add_(0, (c[:, 2] * G[1] + c[:, 1]) * G[0] + c[:, 0], w * up.double())
+    for C, got, flags, name in ((1, out[0], fl[0], "a"), (12, out[1], fl[1], "b")):
+        if name not in form:
+            continue
+        dense = torch.empty(G[2], G[1], G[0], C, device=dev)
+        L.grid_unpack(got, dense, G, C, L.F32)
+        assert float((dense.view(-1, C).double() - ref[C]).abs().max()) <= 1e-5 * float(ref[C].abs().max())
+        assert torch.equal(flags, want)
+
+
+def test_tv_pair_second_trip(L):
+    """Several 64-voxel units per warp: as test_tv_pair_against_single_grids."""
+    test_tv_pair_against_single_grids(L, (160, 131, 150), False)
+
+
+def test_select_second_trip(L):
+    """More rays than the launch's warps take at once (2432 x 2 warps of four)."""
+    rng = np.random.default_rng(9)
+    R, n_draw = 20_011, 5
+    lens = rng.integers(0, 9, R)
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    q = rng.random(int(off[-1])).astype(np.float32) * 0.3
+    ref_sel, ref_n = _select_ref(q, off, n_draw)
+    sel = torch.full((R * n_draw,), 7, dtype=torch.int32, device="cuda")
+    n_sel = torch.full((R,), 7, dtype=torch.int32, device="cuda")
+    L.proposal_select(torch.from_numpy(q).cuda(), torch.from_numpy(off).cuda(), R, n_draw, sel, n_sel)
+    assert np.array_equal(n_sel.cpu().numpy(), ref_n)
+    assert np.array_equal(sel.cpu().numpy().reshape(R, n_draw), ref_sel)
+
+
 def _off_by(t, shift):
     """t's values in a view that starts `shift` elements past a 16-byte boundary."""
     v = torch.empty(t.numel() + shift, dtype=t.dtype, device=t.device)[shift:]

@@ -250,16 +250,15 @@ template <bool kA, bool kB, int kPer>
 __global__ void __launch_bounds__(256) scatter_merge_kernel(
     const float* __restrict__ g_a, float* __restrict__ grid_a, uint8_t* __restrict__ touched_a,
     const float* __restrict__ g_b, float* __restrict__ grid_b, uint8_t* __restrict__ touched_b, TriArgs T,
-    const float* __restrict__ xyz, const int32_t* __restrict__ idx, int64_t n_cap, const int64_t* n_dev) {
+    const float* __restrict__ xyz, const int32_t* __restrict__ idx, int64_t n_cap, const int64_t* n_dev,
+    int64_t crowded_from) {
   __shared__ ScatterStage stages[kB ? 8 : 1];
   ScatterStage& st = stages[kB ? threadIdx.x >> 5 : 0];
   const int64_t n = live_n(n_cap, n_dev);
   const int lane = threadIdx.x & 31;
   const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  // over half a sample per voxel: the density's reductions are spread between
-  // the features' (bursts of them meet in the few sectors they have)
-  const bool crowded = 2 * n > (int64_t)T.g.G[0] * T.g.G[1] * T.g.G[2];
+  const bool crowded = n >= crowded_from;
   for (int64_t j0 = warp0 * kPer; j0 < n; j0 += nwarps * kPer) {
     const int64_t j = j0 + lane;
     const bool valid = lane < kPer && j < n;
@@ -1397,12 +1396,21 @@ template <bool kA, bool kB>
 static void scatter_merge(const float* g_a, float* grid_a, uint8_t* touched_a, const float* g_b, float* grid_b,
                           uint8_t* touched_b, const TriArgs& T, const float* xyz, const int32_t* idx, int64_t n_cap,
                           const int64_t* n_dev, cudaStream_t st) {
+  // Over half a sample per voxel of gradients that stay in L2 (78 MB both), the
+  // density's reductions are spread between the features' (bursts of them meet
+  // in the few sectors they have); else they go out on their own.  Measured on
+  // rays of 48-93 samples, spread and on their own: 64^3 with 0.25 samples a
+  // voxel 13.2 and 12.8 us, 0.5 20.4 and 25.0, 1.0 35.7 and 44.1; 100^3 34 and
+  // 35, 61 and 66, 123 and 131; 128^3 48 and 48, 90 and 91, 183 and 181; 160^3
+  // 92 and 86, 180 and 171, 344 and 334.
+  const int64_t voxels = (int64_t)T.g.G[0] * T.g.G[1] * T.g.G[2];
+  const int64_t crowded_from = voxels <= 1500000 ? voxels / 2 + 1 : INT64_MAX;
   if (n_cap <= kScatterFew)
     scatter_merge_kernel<kA, kB, 8><<<grid_for(4 * n_cap, 256, 16), 256, 0, st>>>(
-        g_a, grid_a, touched_a, g_b, grid_b, touched_b, T, xyz, idx, n_cap, n_dev);
+        g_a, grid_a, touched_a, g_b, grid_b, touched_b, T, xyz, idx, n_cap, n_dev, crowded_from);
   else
     scatter_merge_kernel<kA, kB, 32><<<grid_for(n_cap, 256, 16), 256, 0, st>>>(
-        g_a, grid_a, touched_a, g_b, grid_b, touched_b, T, xyz, idx, n_cap, n_dev);
+        g_a, grid_a, touched_a, g_b, grid_b, touched_b, T, xyz, idx, n_cap, n_dev, crowded_from);
 }
 
 extern "C" int dvgo_sample_grid_bwd(const float* g_out, const dvgo_grid_desc* gd, int32_t C,

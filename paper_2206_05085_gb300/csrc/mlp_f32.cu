@@ -23,7 +23,8 @@
 // form with the X tile built by four warps between two barriers, 127 us with
 // each warp building its own rows (250,000 samples: 248 and 225 us); backward
 // 362, 317 and 300 us (292 with g_k0 on the threads that do not build the
-// input tile; dW1 in 2 x 5 blocks, with fewer wavefronts, was not faster).
+// input tile; dW1 in 2 x 5 blocks, with fewer wavefronts, was not faster).  The
+// backward's 128 registers leave 80 bytes of it in local memory.
 #include "common.cuh"
 #include "mlp_common.cuh"
 

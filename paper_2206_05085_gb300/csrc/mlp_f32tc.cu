@@ -15,9 +15,10 @@
 // input gradient keeps FP32 relative accuracy however small it is.  The
 // weight-gradient products (sums over samples) need one factor for all rows,
 // S, the scale of the largest bound over the CTA's samples: dW2 and dW1 read a
-// second copy of G2's and G1's terms times S / s_s (a row far below the
-// largest loses only terms below FP16's subnormal range, 2^-38 of the largest
-// row).
+// second copy of G2's and G1's terms times S / s_s.  That product is exact while
+// a term stays above 2^-14; below, the hi and the lo term are each rounded to
+// FP16's subnormal step 2^-24 (a row far below the largest loses up to 2^-37
+// of the largest row; a split of the FP32 value itself would lose 2^-38).
 // Every scale is an exact power of two, undone exactly in the epilogues.  A
 // value whose scaled magnitude reaches 2^15 sets DVGO_ERR_RANGE.
 //
@@ -931,7 +932,9 @@ __global__ void __launch_bounds__(kThreads, 1) rgbnet_fwd_tc_kernel(
 // is packed (two FP32 values per instruction), G2 is split once and its
 // second copy formed by multiplying the 16-bit terms.  Measured, 1.9e6
 // samples, FP32 form: 782 us before, 530 us now (393,909 samples: 197 and
-// 142 us; 1003 samples with the partial sums: 31.8 and 25.1 us).
+// 142 us; 1003 samples with the partial sums: 31.8 and 25.1 us).  At the 96
+// registers that 17 warps leave, the FP32 form keeps 116 bytes of its state in
+// local memory, the BF16 form 8.
 //
 // Order per tile t of this CTA (tn = the next one):
 //   compute: wait d2(t) -> G2 of the rows 32 q .. + 15; wait gx(t - 1) ->
@@ -1384,7 +1387,7 @@ __global__ void __launch_bounds__(kThreads, 1) rgbnet_bwd_tc_kernel(
           tc::fence_after_sync();
         }
         st_terms16<Op, false>(sm + bGh, sm + bGl, oh, r0, hl, 1.0f);
-        if (!tiny) {   // (warp-uniform)
+        if (!tiny) {   // (warp-uniform; FP16 terms that fall below 2^-14 are rounded here, BF16 ones are not)
           const uint4 fa = *reinterpret_cast<const uint4*>(fs->fac + r0),
                       fb = *reinterpret_cast<const uint4*>(fs->fac + r0 + 8);
           const uint32_t fac[8] = {fa.x, fa.y, fa.z, fa.w, fb.x, fb.y, fb.z, fb.w};

@@ -68,7 +68,9 @@ class Composite(torch.autograd.Function):
         ctx.save_for_backward(raw, rgb, ray_off, T, n_live)
         ctx.shift, ctx.interval, ctx.bg = shift, interval, bg
         ctx.mark_non_differentiable(n_live)
-        ctx.set_materialize_grads(False)   # an unused output's gradient stays None: no zero tensors are filled
+        # an unused w costs no zero gradient of S entries (an unused color gets
+        # its [R, 3] zeros in backward)
+        ctx.set_materialize_grads(False)
         return color, w, n_live
 
     @staticmethod

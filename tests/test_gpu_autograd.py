@@ -114,6 +114,26 @@ def test_composite_function(O):
     assert np.allclose(fd, host(traw.grad)[idx], rtol=3e-2, atol=3e-3)
 
 
+@pytest.mark.parametrize("used", ["color", "w"])
+def test_composite_one_output_used(O, used):
+    """A loss on the colours alone or on the weights alone: the other output's
+    gradient is absent, as if it were zero."""
+    ops, L = O
+    off, raw, rgb, m, ds = _ragged(11, scale=2.0, bias=1.0)
+    R = len(off) - 1
+    bg = np.array([0.3, 0.6, 0.9], np.float32)
+    shift = float(np.float32(np.log(1 / (1 - 1e-4) - 1)))
+    rng = np.random.default_rng(12)
+    a = rng.normal(size=(R, 3)).astype(np.float32) * (used == "color")
+    b = rng.normal(size=raw.shape).astype(np.float32) * (used == "w")
+    traw, trgb = dev(raw).requires_grad_(True), dev(rgb).requires_grad_(True)
+    color, w, n_live = ops.composite(traw, trgb, dev(off), shift, 0.5, 0.0, bg)
+    (color * dev(a) if used == "color" else w * dev(b)).sum().backward()
+    gr, gc = oracle.composite_bwd(raw, rgb, off, shift, 0.5, 0.0, bg, a, b)
+    assert rel_err(host(traw.grad), gr) < TOL32
+    assert float(np.abs(host(trgb.grad) - gc).max()) <= TOL32 * max(float(np.abs(gc).max()), 1e-30)
+
+
 def test_distortion_function(O):
     ops, L = O
     off, raw, rgb, m, ds = _ragged(4)

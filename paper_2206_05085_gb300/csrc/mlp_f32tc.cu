@@ -1590,11 +1590,15 @@ __global__ void __launch_bounds__(256) partials_reduce_kernel(const float* __res
     const float* src = p < kPartRow ? part + p : part + (size_t)kNumSMs * kPartRow + p - kPartRow;
     const int stride = p < kPartRow ? kPartRow : kOut;
     constexpr int kPer = (kNumSMs + 7) / 8;
-    float v[kPer];   // all of the group's rows in flight at once
+    if (per <= 2) {   // at most 16 rows: 2.4 us, unrolled 3.1 (1003 samples)
+      for (int i = b0; i < b1; ++i) a += __ldg(src + (size_t)i * stride);
+    } else {
+      float v[kPer];   // all of the group's rows in flight at once: 152 rows 4.2 us
 #pragma unroll
-    for (int i = 0; i < kPer; ++i) v[i] = b0 + i < b1 ? __ldg(src + (size_t)(b0 + i) * stride) : 0.0f;
+      for (int i = 0; i < kPer; ++i) v[i] = b0 + i < b1 ? __ldg(src + (size_t)(b0 + i) * stride) : 0.0f;
 #pragma unroll
-    for (int i = 0; i < kPer; ++i) a += v[i];
+      for (int i = 0; i < kPer; ++i) a += v[i];
+    }
   }
   acc[grp][j] = a;
   __syncthreads();
